@@ -1154,10 +1154,13 @@ void split_line_work(const std::vector<SecTask>& tasks, SecLineWork* W, bool mat
     L.mover = tk.mover;
     L.movable = tk.movable;
     L.prepared = tk.prepared;
+    L.q = (uint8_t)Q;
+    std::memcpy(L.bw, tk.bw, sizeof L.bw);
     L.lines = (uint32_t)(tk.size / tk.dim[Q]);
     const uint32_t others = tk.movable & ~(1u << Q);
     const int rm = others == 0 ? -1 : (others & (others - 1)) ? 4 : __builtin_ctz(others);
     const int g = 6 * Q + rm + 1;
+    L.rm = (int16_t)rm;
     for (int q = 0; q < 4; q++) {  // children read through a symmetry: their written-out copies
       if (!(tk.movable >> q & 1) || tk.sym[q] == 0) continue;
       uint8_t cbw[4][2];
@@ -1210,15 +1213,48 @@ std::vector<SecLineTask> rebased_lines(const SecLineWork& W, pp_super* mat) {
   return all;
 }
 
+// Line tasks over ready children laid out for table_line_kernel: one launch
+// whatever the line axes, the blocks that take longest (states walked, times
+// children read) first.  Where the lines alone would give less than about
+// three waves of blocks (two per SM), Q's states are cut into equal ranges;
+// a range pays for the block's tables again, so none is shorter than two
+// steps per warp.
+constexpr uint32_t kTabBlocksWanted = 1024, kTabMinStates = 2 * kTabWarps;
+
+uint32_t lay_out_tables(std::vector<SecLineTask>* tasks) {
+  uint32_t blocks = 0;
+  uint32_t range = 512;  // more than any list of states
+  auto blocks_at = [&](uint32_t states) {
+    uint64_t n = 0;
+    for (const auto& t : *tasks) n += (uint64_t)((t.lines + 31) / 32) * ((t.dim[t.q] + states - 1) / states);
+    return n;
+  };
+  while (range > kTabMinStates && blocks_at(range) < kTabBlocksWanted) range /= 2;
+  auto cost = [](const SecLineTask& t) {
+    uint32_t moves = 0;
+    for (int q = 0; q < 4; q++) moves += 9 - t.bw[q][0] - t.bw[q][1];
+    return (t.dim[t.q] + t.parts - 1) / t.parts * (moves + 2);
+  };
+  for (auto& t : *tasks) t.parts = (uint16_t)((t.dim[t.q] + range - 1) / range);
+  std::stable_sort(tasks->begin(), tasks->end(),
+                   [&](const SecLineTask& a, const SecLineTask& b) { return cost(a) > cost(b); });
+  for (auto& t : *tasks) {
+    t.block0 = blocks;
+    blocks += (t.lines + 31) / 32 * t.parts;
+  }
+  return blocks;
+}
+
+// table_blocks: blocks of the layout of d_lines over ready children (0: raw or
+// prepared children, by groups)
 int launch_line_work(const SecLineWork& W, const SecLineTask* d_lines, const SecTask* d_rest, bool d4, pp_super* out,
-                     pp_stream s, const MatTask* d_mats = nullptr, pp_super* mat = nullptr) {
+                     pp_stream s, const MatTask* d_mats, pp_super* mat, uint32_t table_blocks) {
   int rc = W.mats.empty() ? 0 : launch_materialise(d_mats, (int)W.mats.size(), W.mat_blocks, mat, s);
   if (!rc && !W.rest.empty()) rc = launch_sections(d_rest, (int)W.rest.size(), W.rest_blocks, out, s, d4);
-  // a step's children are all raw, all prepared or all ready
-  const bool ready = !W.all.empty() && W.all[0].prepared == 2;
+  if (!rc && table_blocks) return launch_table_lines(d_lines, (int)W.all.size(), table_blocks, out, s);
   size_t off = 0;
   for (int g = 0; g < kLineGroups && !rc; g++) {
-    rc = launch_section_lines(g / 6, g % 6 - 1, d_lines + off, (int)W.count[g], W.warps[g], out, s, ready);
+    rc = launch_section_lines(g / 6, g % 6 - 1, d_lines + off, (int)W.count[g], W.warps[g], out, s);
     off += W.count[g];
   }
   return rc;
@@ -1238,6 +1274,8 @@ int run_section_lines(const std::vector<SecTask>& tasks, bool d4, pp_super* out,
     if (!e) e = cudaMemcpyAsync(dm, W.mats.data(), W.mats.size() * sizeof(MatTask), cudaMemcpyHostToDevice, s);
   }
   std::vector<SecLineTask> all = rebased_lines(W, mat);
+  // a step's children are all raw, all prepared or all ready
+  const uint32_t table_blocks = !all.empty() && all[0].prepared == 2 ? lay_out_tables(&all) : 0;
   if (!e && !all.empty()) {
     e = cudaMallocAsync((void**)&dl, all.size() * sizeof(SecLineTask), s);
     if (!e) e = cudaMemcpyAsync(dl, all.data(), all.size() * sizeof(SecLineTask), cudaMemcpyHostToDevice, s);
@@ -1246,7 +1284,7 @@ int run_section_lines(const std::vector<SecTask>& tasks, bool d4, pp_super* out,
     e = cudaMallocAsync((void**)&dr, W.rest.size() * sizeof(SecTask), s);
     if (!e) e = cudaMemcpyAsync(dr, W.rest.data(), W.rest.size() * sizeof(SecTask), cudaMemcpyHostToDevice, s);
   }
-  int rc = e ? (int)e : launch_line_work(W, dl, dr, d4, out, s, dm, mat);
+  int rc = e ? (int)e : launch_line_work(W, dl, dr, d4, out, s, dm, mat, table_blocks);
   if (dl) cudaFreeAsync(dl, s);
   if (dr) cudaFreeAsync(dr, s);
   if (dm) cudaFreeAsync(dm, s);
@@ -1547,6 +1585,7 @@ struct pp_slice_plan {
   // thread per board (2)
   bool has_slines = false, slines = false;
   SecLineWork sw;
+  uint32_t table_blocks = 0;  // of the layout of d_sl when the children are ready
   SecLineTask* d_sl = nullptr;
   SecTask* d_srest = nullptr;
   MatTask* d_mats = nullptr;  // D4: children written out in their own layout at each run
@@ -1723,7 +1762,8 @@ int pp_slice_plan_run(pp_slice_plan* P, pp_stream s) {
     rc = P->ntasks ? launch_sections(P->d_tasks, P->ntasks, P->blocks, P->out, s, true) : 0;
     if (!rc && !P->lw.all.empty()) rc = launch_line35_work(P->lw, P->d_ltasks, P->tmp, P->out, s);
   } else if (P->slines) {
-    rc = launch_line_work(P->sw, P->d_sl, P->d_srest, P->d4, P->out, s, P->d_mats, P->mat);
+    rc = launch_line_work(P->sw, P->d_sl, P->d_srest, P->d4, P->out, s, P->d_mats, P->mat,
+                          P->prepared == 2 ? P->table_blocks : 0);
   } else if (P->persistent == 1) {
     rc = launch_sections_persistent(P->d_tasks, P->ntasks, P->blocks, P->out, P->d_counter,
                                     persistent_section_blocks(P->ctas_per_sm, P->d4), s, P->d4);
@@ -1787,6 +1827,7 @@ int pp_slice_plan_set_prepared(pp_slice_plan* P, int prepared) {
   cudaError_t e = cudaSuccess;
   if (P->d_sl && !P->sw.all.empty()) {
     auto all = rebased_lines(P->sw, P->mat);
+    if (prepared == 2) P->table_blocks = lay_out_tables(&all);
     e = cudaMemcpy(P->d_sl, all.data(), all.size() * sizeof(SecLineTask), cudaMemcpyHostToDevice);
   }
   if (!e && P->d_srest && !P->sw.rest.empty())

@@ -16,6 +16,9 @@ namespace pp {
 constexpr int kQStates = 19683;   // 3^9 patterns of one quadrant
 constexpr int kMinStates = 4995;  // rotation classes of one quadrant
 constexpr int kFormWords = 12;    // words per (quadrant, pattern) five-table entry
+constexpr int kMoveSlots = 12;    // entries per state of the move lists (9 used; 8-byte aligned)
+constexpr int kCoverBytes = 20;   // room for every line through a quadrant, by words
+constexpr int kLinesPerQuad = 17; // five-in-a-row lines that touch one quadrant
 constexpr int kMaxEmpty = 16;     // deepest midgame fill table: 3^16 entries
 // sum over c = 0..8 of the 16-bit values with at most c bits set
 constexpr int kCappedSubsets = 90683;
@@ -87,6 +90,23 @@ struct HostTables {
   // so the subsets of the first k slots with at most c of them are the
   // block's first sum over j <= c of C(k, j) entries
   uint16_t subsets[kCappedSubsets];
+  // pattern tables of the line kernels (see table_lines): the 32 lines in a
+  // fixed order; nibble l % 8 of lsets[q][x][l / 8] is S_{l,q}(x) (0xF when
+  // line l misses q); ltouch[q]: the lines that touch q.  The 512 patterns y
+  // ordered by number of stones, then value (those with n stones start at
+  // yoff[n]): lcover[q][place of y] lists the lines through q whose cells of
+  // q lie inside y, a byte each: s for the s-th line touching q (in line
+  // order), kLinesPerQuad after the last
+  uint32_t lsets[4][512][4];
+  uint32_t ltouch[4];
+  uint8_t lcover[4][512][kCoverBytes];
+  uint16_t yoff[11];
+  // per state i and colour (black, white): byte t = the place, among the
+  // patterns of as many stones, of the colour's pattern turned t times
+  uint32_t yrank[kMinStates][2];
+  // per mover colour and state: the child's rank | turn << 12 for each empty
+  // cell in increasing order
+  uint16_t qmoves[2][kMinStates][kMoveSlots];
 };
 
 const HostTables& host_tables();
@@ -139,6 +159,12 @@ struct DeviceTables {
   const uint32_t* qsorted;  // [2][kMinStates][4]
   const uint16_t* dmin;     // [8][kMinStates]
   const uint16_t* subsets;  // [kCappedSubsets]
+  const uint32_t* lsets;    // [4][512][4]
+  const uint32_t* lcover;   // [4][512][kCoverBytes / 4]
+  const uint32_t* yrank;    // [kMinStates][2]
+  const uint16_t* qmoves;   // [2][kMinStates][kMoveSlots]
+  uint32_t ltouch[4];
+  uint16_t yoff[11];
   int qoff[10][10];
   int qdim[10][10];
 };
@@ -301,8 +327,16 @@ struct SecLineTask {
   uint8_t mover;             // 1 black, 2 white
   uint8_t movable;           // bit q: quadrant q has an empty cell
   uint8_t prepared;          // 1: child values in prepared form (pp_prepare_children)
-  uint8_t pad;
+  uint8_t q;                 // the line axis Q
+  uint8_t bw[4][2];          // stones per quadrant
+  // table_line_kernel: a block of kTabWarps warps owns 32 lines and one of
+  // `parts` equal ranges of Q's states
+  uint32_t block0;           // first block of this task (tasks in block order)
+  uint16_t parts;
+  int16_t rm;                // the one other quadrant with empty cells (0..3, not q), -1 none, 4 several
 };
+constexpr int kTabWarps = 8;
+constexpr int kTabEntries = 126;  // most patterns with the same number of stones, C(9, 4)
 
 // ---------------------------------------------------------------------------
 // Kernel launchers (pp_kernels.cu).  All return a cudaError_t value.
@@ -361,7 +395,9 @@ int launch_materialise(const MatTask* d_tasks, int ntasks, uint32_t blocks, pp_s
 
 // rm: the one other quadrant with empty cells (0..3, not q), -1 none, 4 any
 int launch_section_lines(int q, int rm, const SecLineTask* d_tasks, int ntasks, uint32_t warps, pp_super* d_out,
-                         pp_stream s, bool ready = false);
+                         pp_stream s);
+// ready children, any mix of line axes
+int launch_table_lines(const SecLineTask* d_tasks, int ntasks, uint32_t blocks, pp_super* d_out, pp_stream s);
 int launch_five_masks(const uint64_t* d_boards, int n, uint64_t* d_out, pp_stream s);
 int launch_rmax(const pp_super* d_in, int n, pp_super* d_out, pp_stream s);
 int launch_shift(const pp_super* d_in, int n, int q, int u, pp_super* d_out, pp_stream s);

@@ -11,6 +11,7 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 
 #include "pp_internal.h"
 
@@ -37,8 +38,8 @@
 #ifndef PP_SLINE_MINB
 #define PP_SLINE_MINB 2  // section line kernel
 #endif
-#ifndef PP_SLINE_READY_MINB
-#define PP_SLINE_READY_MINB 3  // section line kernel over ready children (80 registers)
+#ifndef PP_TAB_MINB
+#define PP_TAB_MINB 2  // pattern-table line kernel (128 registers, see table_line_kernel)
 #endif
 #ifndef PP_SLINE_WARPS
 #define PP_SLINE_WARPS 8  // warps per block of the section line kernel
@@ -511,6 +512,13 @@ __device__ __forceinline__ int find_block_owner(const T* __restrict__ d, int n, 
 // the load freely.
 __device__ __forceinline__ void ld256_nc(const void* p, uint32_t r[8]) {
   asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "l"(p));
+}
+// The same, kept in program order with the stores and other such loads: for
+// loads meant to be in flight during the work written after them.
+__device__ __forceinline__ void ld256_nc_early(const void* p, uint32_t r[8]) {
+  asm volatile("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "l"(p));
 }
@@ -1580,7 +1588,8 @@ __global__ void __launch_bounds__(kLineWarps * 32, PP_LINE_MINB)
 // Q's states in order.  Q's pattern is then the same in every lane, so its
 // forms, its moves' child ranks and turns are uniform.  The five-in-a-row and
 // immediate-win terms of the lines that miss Q are computed once per line
-// (K); each step evaluates only the lines through Q.
+// (K); each step evaluates only the lines through Q.  For raw and prepared
+// children (ready ones carry the immediate wins: table_line_kernel).
 // ---------------------------------------------------------------------------
 // Which fixed quadrants can take a move, known at compile time: RM = -1
 // none, 0..3 exactly that one, 4 any (read from the task).
@@ -1620,12 +1629,8 @@ __device__ __forceinline__ void line_moves(const SecLineTask& tk, const uint32_t
 constexpr int kSecLineColdWords = 3 * kLineUsedWords + 24;  // + the K terms (Kc, Ki, Ko)
 constexpr size_t kSecLineSmem = sizeof(uint32_t) * kSecLineWarps * 32 * kSecLineColdWords;
 
-// READY: the children are ready records (pp_prepare_children_ready), which
-// carry each child's five-in-a-row set of this slice's mover: the OR over
-// the moves already holds the immediate-win mask, so no line is evaluated
-// with one more stone.
-template <int Q, int RM, bool READY>
-__global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MINB : PP_SLINE_MINB)
+template <int Q, int RM>
+__global__ void __launch_bounds__(kSecLineWarps * 32, PP_SLINE_MINB)
     section_line_kernel(const SecLineTask* __restrict__ tasks, int ntasks, pp_super* __restrict__ out) {
   extern __shared__ uint32_t sline_cold[];
   uint32_t* mycold = sline_cold + threadIdx.x;  // word i at mycold[i * blockDim]
@@ -1656,7 +1661,7 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
     pc[q] = c == 1 ? b : w;
     load_forms(q, pc[q], fc[q]);
     load_forms(q, c == 1 ? w : b, fo[q]);
-    if (!READY && fixed_movable<RM>(tk, q)) {
+    if (fixed_movable<RM>(tk, q)) {
       for (uint32_t em = ~(b | w) & 0x1FFu; em; em &= em - 1) {
         uint32_t g[kFormWords];
         load_forms(q, pc[q] | 1u << (__ffs(em) - 1), g);
@@ -1666,11 +1671,8 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
     }
     obase += (uint64_t)idx[q] * tk.stride[q];
   }
-  uint32_t Kc[8], Ki[8] = {0, 0, 0, 0, 0, 0, 0, 0}, Ko[8];
-  if (READY)
-    five_mask(fc, Kc);
-  else
-    eval_all_fives<true>(fc, fi, Kc, Ki);  // quadrant Q's forms are zero: the lines missing Q
+  uint32_t Kc[8], Ki[8], Ko[8];
+  eval_all_fives<true>(fc, fi, Kc, Ki);  // quadrant Q's forms are zero: the lines missing Q
   five_mask(fo, Ko);
   // park the form words the steps read; the registers are then free
 #pragma unroll
@@ -1680,13 +1682,13 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
       if (line_word_used<Q>(q, w)) {
         const int k = line_word_slot<Q>(q, w);
         cold_at(k) = fc[q][w];
-        if (!READY) cold_at(kLineUsedWords + k) = fi[q][w];
+        cold_at(kLineUsedWords + k) = fi[q][w];
         cold_at(2 * kLineUsedWords + k) = fo[q][w];
       }
 #pragma unroll
   for (int i = 0; i < 8; i++) {
     cold_at(3 * kLineUsedWords + i) = Kc[i];
-    if (!READY) cold_at(3 * kLineUsedWords + 8 + i) = Ki[i];
+    cold_at(3 * kLineUsedWords + 8 + i) = Ki[i];
     cold_at(3 * kLineUsedWords + 16 + i) = Ko[i];
   }
 
@@ -1711,7 +1713,7 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
         const bool used = line_word_used<Q>(q, w);
         const int k = used ? line_word_slot<Q>(q, w) : 0;
         fc[q][w] = used ? cold_at(k) : 0u;
-        fi[q][w] = used && !READY ? cold_at(kLineUsedWords + k) : 0u;
+        fi[q][w] = used ? cold_at(kLineUsedWords + k) : 0u;
         fo[q][w] = used ? cold_at(2 * kLineUsedWords + k) : 0u;
       }
     const uint32_t cq = __ldg(c_tab.qlist + tk.qoff[Q] + p);  // uniform across the warp
@@ -1722,18 +1724,14 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
     load_forms(Q, c == 1 ? wq : bq, fo[Q]);
 #pragma unroll
     for (int x = 0; x < kFormWords; x++) fi[Q][x] = 0;
-    uint32_t Hc[8], Hi[8] = {0, 0, 0, 0, 0, 0, 0, 0}, Ho[8], unused[8];
-    if (READY) {
-      eval_fives<false, Q>(fc, fc, Hc, unused);
-    } else {
-      for (uint32_t em = eq; em; em &= em - 1) {
-        uint32_t g[kFormWords];
-        load_forms(Q, pcq | 1u << (__ffs(em) - 1), g);
+    for (uint32_t em = eq; em; em &= em - 1) {
+      uint32_t g[kFormWords];
+      load_forms(Q, pcq | 1u << (__ffs(em) - 1), g);
 #pragma unroll
-        for (int x = 0; x < kFormWords; x++) fi[Q][x] |= g[x];
-      }
-      eval_fives<true, Q>(fc, fi, Hc, Hi);
+      for (int x = 0; x < kFormWords; x++) fi[Q][x] |= g[x];
     }
+    uint32_t Hc[8], Hi[8], Ho[8], unused[8];
+    eval_fives<true, Q>(fc, fi, Hc, Hi);
     eval_fives<false, Q>(fo, fo, Ho, unused);
     uint32_t AW[8] = {0, 0, 0, 0, 0, 0, 0, 0}, AN[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     // moves in Q: child rank and turn uniform
@@ -1755,11 +1753,462 @@ __global__ void __launch_bounds__(kSecLineWarps * 32, READY ? PP_SLINE_READY_MIN
 #pragma unroll
     for (int w = 0; w < 8; w++) {
       Fc[w] = cold_at(3 * kLineUsedWords + w) | Hc[w];
-      I[w] = READY ? 0u : cold_at(3 * kLineUsedWords + 8 + w) | Hi[w];
+      I[w] = cold_at(3 * kLineUsedWords + 8 + w) | Hi[w];
       Fo[w] = cold_at(3 * kLineUsedWords + 16 + w) | Ho[w];
     }
     combine(Fc, Fo, I, AW, AN, W, N, tk.prepared != 0);
     if (active) store_super32(out + obase + (uint64_t)p * tk.stride[Q], W, N);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Section lines over ready children, with pattern tables.  A line fixes three
+// quadrants and walks the fourth, Q.  At quadrant Q's turn t the set of the
+// other three quadrants' turns with a five is
+//     G(y) = K | OR over the lines l through Q with l's cells of Q inside y of M_l,
+// y = Q's pattern of that colour turned t times, K the lines missing Q and
+// M_l the product of l's turn sets in the fixed quadrants (64 bits each).  So
+// a board's 256-bit set F is four table entries G(y_0..y_3), and the
+// states of Q share the table: C(9, stones) entries per colour, at most 126,
+// for up to 420 states.  One block owns 32 lines; its warps build both
+// colours' tables in shared memory, [entry][line], then divide Q's states
+// among them.
+//
+// Evaluating the lines of every board took about 550 instructions a board and
+// left the integer pipe the bound; with the tables a board takes about 300
+// (its share of the tables included, a seventh of the time).  What bounds it
+// now is the integer pipe (45-55%) and the latency of the children's loads at
+// 16 warps per SM (two blocks of 74 KB; three at 80 registers spill: 12.3
+// against 10.7 ms for the step below).  One launch takes every line axis and
+// shape, blocks of the most work first: a launch per shape ended each on a
+// few long walks.  Measured, 300 million boards of D4 slice 34 with the
+// ready pass: 20.5 -> 10.7 ms; 60 million of slice 33 through its cone,
+// where most shapes had fewer lines than fill the device: 16.3 -> 3.5 ms.
+// ---------------------------------------------------------------------------
+
+// A 64-bit set over the fixed quadrants' turns, in the order spread_turns<Q>
+// reads: index bit 5 selects the word (.x, .y), bits 0-4 the position.  For
+// Q = 3 and 2 the index is g_a + 4 g_b + 16 g_c (a < b < c the fixed
+// quadrants); for Q = 1 and 0 the output word (g3 & 1, g2 >> 1) is moved
+// next to the low bits, so that spreading is a transpose of 4 x 4 nibbles or
+// bits.  set_bit(k, hi): where the low or high bit of the k-th fixed
+// quadrant's turn sits.
+template <int Q>
+__host__ __device__ constexpr int set_bit(int k, bool hi) {
+  if (Q == 1 && k > 0) return k == 1 ? (hi ? 2 : 4) : (hi ? 5 : 3);
+  if (Q == 0) return k == 0 ? (hi ? 3 : 2) : k == 1 ? (hi ? 0 : 4) : (hi ? 5 : 1);
+  return 2 * k + (hi ? 1 : 0);
+}
+// The positions where the k-th fixed quadrant's turn is t.
+template <int Q>
+__host__ __device__ constexpr uint64_t turn_positions(int k, int t) {
+  uint64_t m = 0;
+  for (int i = 0; i < 64; i++)
+    if ((i >> set_bit<Q>(k, false) & 1) == (t & 1) && (i >> set_bit<Q>(k, true) & 1) == (t >> 1)) m |= 1ull << i;
+  return m;
+}
+
+// The 256-bit set whose slice at quadrant Q's turn t is g[t].
+template <int Q>
+__device__ __forceinline__ void spread_turns(const uint2 (&g)[4], uint32_t F[8]) {
+  if constexpr (Q == 3) {
+#pragma unroll
+    for (int t = 0; t < 4; t++) F[2 * t] = g[t].x, F[2 * t + 1] = g[t].y;
+  } else if constexpr (Q == 2) {
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      F[h] = __byte_perm(g[2 * h].x, g[2 * h + 1].x, 0x5410);
+      F[h + 2] = __byte_perm(g[2 * h].x, g[2 * h + 1].x, 0x7632);
+      F[h + 4] = __byte_perm(g[2 * h].y, g[2 * h + 1].y, 0x5410);
+      F[h + 6] = __byte_perm(g[2 * h].y, g[2 * h + 1].y, 0x7632);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      const uint32_t a0 = j ? g[0].y : g[0].x, a1 = j ? g[1].y : g[1].x;
+      const uint32_t a2 = j ? g[2].y : g[2].x, a3 = j ? g[3].y : g[3].x;
+      if constexpr (Q == 1) {  // 4 x 4 transposes of nibbles
+        constexpr uint32_t m = 0x0F0F0F0Fu;
+        const uint32_t t0 = (a0 & m) | ((a1 << 4) & ~m), t1 = ((a0 >> 4) & m) | (a1 & ~m);
+        const uint32_t u0 = (a2 & m) | ((a3 << 4) & ~m), u1 = ((a2 >> 4) & m) | (a3 & ~m);
+        F[4 * j] = __byte_perm(t0, u0, 0x6240);
+        F[4 * j + 1] = __byte_perm(t1, u1, 0x6240);
+        F[4 * j + 2] = __byte_perm(t0, u0, 0x7351);
+        F[4 * j + 3] = __byte_perm(t1, u1, 0x7351);
+      } else {  // of bits
+        constexpr uint32_t m = 0x55555555u, n = 0x33333333u;
+        const uint32_t t0 = (a0 & m) | ((a1 << 1) & ~m), t1 = ((a0 >> 1) & m) | (a1 & ~m);
+        const uint32_t u0 = (a2 & m) | ((a3 << 1) & ~m), u1 = ((a2 >> 1) & m) | (a3 & ~m);
+        F[4 * j] = (t0 & n) | ((u0 << 2) & ~n);
+        F[4 * j + 1] = (t1 & n) | ((u1 << 2) & ~n);
+        F[4 * j + 2] = ((t0 >> 2) & n) | (u0 & ~n);
+        F[4 * j + 3] = ((t1 >> 2) & n) | (u1 & ~n);
+      }
+    }
+  }
+}
+
+constexpr int kTabMoves = 27;  // the most moves in the three fixed quadrants
+static_assert(kTabMoves <= 2 * (kLinesPerQuad + 1), "the move list reuses the line products' room");
+
+struct TableSmem {
+  uint2 K[2][32];                     // per colour and lane: the lines missing Q
+  uint2 M[2][kLinesPerQuad + 1][32];  // M_l of the lines through Q, then zero; later the fixed quadrants' moves
+  uint2 S[3][16];                     // a turn set of the k-th fixed quadrant as a set of positions
+  uint2 G[2][kTabEntries][32];        // the mover's table, the opponent's
+};
+
+// One table (8 words) of a child turned u quarter turns along axis R, any u
+// per lane.
+template <int R>
+__device__ __forceinline__ void turn_table(uint32_t x[8], uint32_t u) {
+  if constexpr (R == 2) {  // the word pair (g2 = 0, 1), (2, 3) as eight bytes, rotated by 2u
+    const uint32_t sel = u == 0 ? 0x3210u : u == 1 ? 0x5432u : u == 2 ? 0x7654u : 0x1076u;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      const uint32_t lo = x[2 * j], hi = x[2 * j + 1];
+      x[2 * j] = __byte_perm(lo, hi, sel);
+      x[2 * j + 1] = __byte_perm(hi, lo, sel);
+    }
+  } else {
+    shift_axis<R>(x, u);
+  }
+}
+
+// The table of one board from its sets and x, the AND over its children's
+// tables: not-lose from their win tables, win from their not-lose tables.
+__device__ __forceinline__ void table_combine(const uint32_t Fc[8], const uint32_t Fo[8], uint32_t notlose,
+                                              uint32_t x[8]) {
+#pragma unroll
+  for (int w = 0; w < 8; w++) {
+    const uint32_t own = Fc[w] & (notlose | ~Fo[w]);
+    x[w] = own | (~Fo[w] & ~x[w]);
+  }
+}
+
+template <int Q>
+__device__ __forceinline__ void table_sets(const TableSmem& sm, uint32_t place, uint32_t ranks, int colour, int half,
+                                           uint32_t F[8]) {
+  uint2 g[4];
+#pragma unroll
+  for (int t = 0; t < 4; t++)  // entry byte t of ranks, this lane's column: one byte permute is the whole offset
+    g[t] = *reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(&sm.G[colour][0][16 * half]) +
+                                           __byte_perm(ranks, place, 0x5504u + 16 * t));
+  spread_turns<Q>(g, F);
+}
+
+// Pairs of lanes share lines: lane l handles one table (its parity) of lines
+// l / 2 and l / 2 + 16, so that a warp's loads and stores of one line set
+// cover 1 KB without gaps (64-byte records read half by half, a lane each,
+// took twice the L1 wavefronts).
+template <int Q, int RM>
+__device__ __forceinline__ void table_walk(const SecLineTask& tk, const TableSmem& sm, int warp, uint32_t s0,
+                                           uint32_t s1, int qmoves, uint64_t obase, const pp_super* qbase,
+                                           uint32_t lines_left, pp_super* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t c = tk.mover;
+  const uint32_t h = lane & 1, la = lane >> 1;
+  const uint32_t notlose = h ? 0u : 0xFFFFFFFFu;  // children's win tables make not-lose
+  const bool va = la < lines_left, vb = la + 16 < lines_left;
+  char* oa = reinterpret_cast<char*>(out + __shfl_sync(0xFFFFFFFFu, obase, la)) + 32 * (1 - h);
+  char* ob = reinterpret_cast<char*>(out + __shfl_sync(0xFFFFFFFFu, obase, la + 16)) + 32 * (1 - h);
+  const uint64_t q64 = reinterpret_cast<uint64_t>(qbase);
+  const char* qa = reinterpret_cast<const char*>(__shfl_sync(0xFFFFFFFFu, q64, la)) + 32 * h;
+  const char* qb = reinterpret_cast<const char*>(__shfl_sync(0xFFFFFFFFu, q64, la + 16)) + 32 * h;
+  const uint64_t* mva = reinterpret_cast<const uint64_t*>(&sm.M[0][0][0]) + la;  // moves: [move][line]
+  const uint32_t cq = (uint32_t)tk.cstride[Q][Q], sq = tk.stride[Q];
+  const uint32_t* __restrict__ sorted = c_tab.qsorted + ((c - 1) * kMinStates + tk.qoff[Q]) * 4 + 1;
+  const uint16_t* __restrict__ mvq = c_tab.qmoves + ((c - 1) * kMinStates + tk.qoff[Q]) * kMoveSlots;
+  const uint2* __restrict__ yrank = reinterpret_cast<const uint2*>(c_tab.yrank) + tk.qoff[Q];
+  const uint32_t place = la * 8;
+
+  // Q's states, one after the other over the block's warps; 32 steps' state
+  // numbers, table places and first moves are read at once, a lane each
+  const uint32_t steps = s0 + warp < s1 ? (s1 - s0 - warp + kTabWarps - 1) / kTabWarps : 0;
+  uint32_t sp = 0, src = 0, sro = 0, smv = 0;
+  auto q_move = [&](uint32_t v, uint32_t a[8], uint32_t b[8]) {
+    const uint64_t at = (uint64_t)(v & 0xFFFu) * cq * sizeof(pp_super);
+    ld256_nc_early(qa + at, a);
+    ld256_nc_early(qb + at, b);
+  };
+  auto fixed_move = [&](int R, int f, uint32_t p, uint32_t a[8], uint32_t b[8]) {
+    const uint64_t ma = mva[f * 32], mb = mva[f * 32 + 16];
+    const uint64_t at = (uint64_t)p * tk.cstride[R][Q] * sizeof(pp_super) + 32 * h;
+    ld256_nc_early(reinterpret_cast<const char*>(ma & ~(uint64_t)31) + at, a);
+    ld256_nc_early(reinterpret_cast<const char*>(mb & ~(uint64_t)31) + at, b);
+  };
+  auto fold = [](uint32_t a[8], uint32_t b[8], const uint32_t c[8], const uint32_t d[8]) {
+#pragma unroll
+    for (int w = 0; w < 8; w++) a[w] &= c[w], b[w] &= d[w];
+  };
+  // A step's first two children: Q's first move, then Q's second or the one
+  // other quadrant's first.
+  auto fetch = [&](uint32_t step, uint32_t xa[8], uint32_t xb[8], uint32_t ya[8], uint32_t yb[8]) {
+    if ((step & 31) == 0) {
+      const uint32_t k = s0 + warp + kTabWarps * (step + lane);
+      if (k < s1) {
+        // one empty cell: in the order of the child's rank, so that the
+        // warps read the same child at about the same time (L1)
+        sp = qmoves == 1 ? __ldg(sorted + 4 * k) >> 16 : k;
+        const uint2 y = __ldg(yrank + sp);
+        src = c == 1 ? y.x : y.y;
+        sro = c == 1 ? y.y : y.x;
+        smv = __ldg(reinterpret_cast<const uint32_t*>(mvq + sp * kMoveSlots));
+      }
+    }
+    const uint32_t mv = __shfl_sync(0xFFFFFFFFu, smv, step & 31);
+    q_move(mv, xa, xb);
+    if constexpr (RM >= 0 && RM < 4)
+      fixed_move(RM, 0, __shfl_sync(0xFFFFFFFFu, sp, step & 31), ya, yb);
+    else if (qmoves > 1)
+      q_move(mv >> 16, ya, yb);
+  };
+  const uint32_t ua0 = RM >= 0 ? (uint32_t)mva[0] & 3u : 0u, ub0 = RM >= 0 ? (uint32_t)mva[16] & 3u : 0u;
+  auto walk_step = [&](uint32_t step) {
+    uint32_t xa[8], xb[8], ya[8], yb[8];
+    fetch(step, xa, xb, ya, yb);
+    const uint32_t p = __shfl_sync(0xFFFFFFFFu, sp, step & 31), mv = __shfl_sync(0xFFFFFFFFu, smv, step & 31);
+    const uint32_t rc = __shfl_sync(0xFFFFFFFFu, src, step & 31), ro = __shfl_sync(0xFFFFFFFFu, sro, step & 31);
+    uint32_t Fc[8], Fo[8];
+    table_sets<Q>(sm, place, rc, 0, 0, Fc);
+    table_sets<Q>(sm, place, ro, 1, 0, Fo);
+    if (mv >> 12 & 3u) {  // uniform
+      turn_table<Q>(xa, mv >> 12 & 3u);
+      turn_table<Q>(xb, mv >> 12 & 3u);
+    }
+    if constexpr (RM >= 0 && RM < 4) {
+      turn_table<RM>(ya, ua0);
+      turn_table<RM>(yb, ub0);
+      fold(xa, xb, ya, yb);
+      const int empties = 9 - tk.bw[RM][0] - tk.bw[RM][1];
+      for (int f = 1; f < empties; f++) {
+        fixed_move(RM, f, p, ya, yb);
+        turn_table<RM>(ya, (uint32_t)mva[f * 32] & 3u);
+        turn_table<RM>(yb, (uint32_t)mva[f * 32 + 16] & 3u);
+        fold(xa, xb, ya, yb);
+      }
+      if (qmoves > 1) q_move(mv >> 16, ya, yb);
+    }
+    if (qmoves > 1) {
+      if (mv >> 28) {
+        turn_table<Q>(ya, mv >> 28);
+        turn_table<Q>(yb, mv >> 28);
+      }
+      fold(xa, xb, ya, yb);
+      for (int i = 2; i < qmoves; i++) {
+        const uint32_t v = __ldg(mvq + p * kMoveSlots + i);
+        q_move(v, ya, yb);
+        turn_table<Q>(ya, v >> 12);
+        turn_table<Q>(yb, v >> 12);
+        fold(xa, xb, ya, yb);
+      }
+    }
+    if constexpr (RM == 4) {
+      int f = 0;
+      auto quadrant = [&](auto Rc) {
+        constexpr int R = decltype(Rc)::value;
+        if constexpr (R != Q) {
+          const int empties = 9 - tk.bw[R][0] - tk.bw[R][1];
+          for (int i = 0; i < empties; i++, f++) {
+            fixed_move(R, f, p, ya, yb);
+            turn_table<R>(ya, (uint32_t)mva[f * 32] & 3u);
+            turn_table<R>(yb, (uint32_t)mva[f * 32 + 16] & 3u);
+            fold(xa, xb, ya, yb);
+          }
+        }
+      };
+      quadrant(std::integral_constant<int, 0>{});
+      quadrant(std::integral_constant<int, 1>{});
+      quadrant(std::integral_constant<int, 2>{});
+      quadrant(std::integral_constant<int, 3>{});
+    }
+    table_combine(Fc, Fo, notlose, xa);
+    const uint64_t at = (uint64_t)p * sq * sizeof(pp_super);
+    if (va) st256(oa + at, xa);
+    table_sets<Q>(sm, place, rc, 0, 1, Fc);
+    table_sets<Q>(sm, place, ro, 1, 1, Fo);
+    table_combine(Fc, Fo, notlose, xb);
+    if (vb) st256(ob + at, xb);
+  };
+  for (uint32_t step = 0; step < steps; step++) walk_step(step);
+}
+
+template <int Q>
+__device__ __forceinline__ void table_lines(const SecLineTask& tk, uint32_t group, uint32_t part, TableSmem& sm,
+                                            pp_super* __restrict__ out) {
+  constexpr int A = Q == 0 ? 1 : 0, B = Q <= 1 ? 2 : 1, C = Q == 3 ? 2 : 3;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0);
+  const uint32_t line = group * 32 + lane;
+  const uint32_t c = tk.mover;
+  if (threadIdx.x < 48) {
+    const int k = threadIdx.x / 16, set = threadIdx.x % 16;
+    uint64_t m = 0;
+#pragma unroll
+    for (int t = 0; t < 4; t++)
+      if (set >> t & 1)
+        m |= k == 0 ? turn_positions<Q>(0, t) : k == 1 ? turn_positions<Q>(1, t) : turn_positions<Q>(2, t);
+    sm.S[k][set] = make_uint2((uint32_t)m, (uint32_t)(m >> 32));
+  }
+  const int nc = tk.bw[Q][c - 1], no = tk.bw[Q][2 - c];
+  const int yc = c_tab.yoff[nc + 1] - c_tab.yoff[nc], yo = c_tab.yoff[no + 1] - c_tab.yoff[no];
+  // the first four lines inside each of this warp's table entries: lane i
+  // holds those of the warp's i-th entry of either colour (at most 16)
+  constexpr int kPerColour = 16;
+  static_assert(kPerColour * kTabWarps >= kTabEntries, "every entry has a warp and a lane");
+  const uint32_t* __restrict__ cover = c_tab.lcover + Q * 512 * (kCoverBytes / 4);
+  uint32_t covers = 0;
+  {
+    const int t = warp + kTabWarps * (lane % kPerColour), col = lane / kPerColour;
+    if (t < (col ? yo : yc)) covers = __ldg(cover + (c_tab.yoff[col ? no : nc] + t) * (kCoverBytes / 4));
+  }
+  uint32_t idx[4] = {0, 0, 0, 0};
+  uint32_t r = line < tk.lines ? line : 0;
+  uint64_t obase = tk.out;
+  // this warp's four lines' turn sets in the fixed quadrants, both colours
+  uint32_t sc[4], so[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    if (q == Q) continue;
+    idx[q] = r % tk.dim[q];
+    r /= tk.dim[q];
+    const uint32_t x = __ldg(c_tab.qline + 2 * (tk.qoff[q] + idx[q])), b = x & 0x1FFu, w = x >> 9;
+    sc[q] = __ldg(c_tab.lsets + (q * 512 + (c == 1 ? b : w)) * 4 + (warp >> 1)) >> (16 * (warp & 1));
+    so[q] = __ldg(c_tab.lsets + (q * 512 + (c == 1 ? w : b)) * 4 + (warp >> 1)) >> (16 * (warp & 1));
+    obase += (uint64_t)idx[q] * tk.stride[q];
+  }
+  const uint32_t touch = c_tab.ltouch[Q];
+  static_assert(kTabWarps * 4 == 32, "four lines per warp");
+  __syncthreads();
+#pragma unroll
+  for (int col = 0; col < 2; col++) {
+    uint2 k = make_uint2(0, 0);
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const uint32_t (&s)[4] = col ? so : sc;
+      const uint2 a = sm.S[0][s[A] >> (4 * i) & 15u], b = sm.S[1][s[B] >> (4 * i) & 15u];
+      const uint2 d = sm.S[2][s[C] >> (4 * i) & 15u];
+      const uint2 m = make_uint2(a.x & b.x & d.x, a.y & b.y & d.y);
+      const int l = warp * 4 + i;
+      if (touch >> l & 1u)
+        sm.M[col][__popc(touch & ((1u << l) - 1u))][lane] = m;
+      else
+        k.x |= m.x, k.y |= m.y;
+    }
+    if (k.x) atomicOr(&sm.K[col][lane].x, k.x);
+    if (k.y) atomicOr(&sm.K[col][lane].y, k.y);
+  }
+  __syncthreads();
+  // both colours' tables: two lines at a time, the second pair where there
+  // are more than two (a third of the entries), the rest one by one (few)
+#pragma unroll
+  for (int col = 0; col < 2; col++) {
+    const uint2 k = sm.K[col][lane];
+    const int entries = col ? yo : yc;
+    const char* Mc = reinterpret_cast<const char*>(&sm.M[col][0][lane]);
+    auto product = [&](uint32_t offset) { return *reinterpret_cast<const uint2*>(Mc + offset); };
+    for (int t = warp, i = col * kPerColour; t < entries; t += kTabWarps, i++) {
+      const uint32_t list = __shfl_sync(0xFFFFFFFFu, covers, i);  // a byte times 256 is an entry's offset
+      const uint2 m0 = product(__byte_perm(list, 0, 0x4404)), m1 = product(__byte_perm(list, 0, 0x4414));
+      uint2 g = make_uint2(k.x | m0.x | m1.x, k.y | m0.y | m1.y);
+      if ((list >> 16 & 0xFFu) != kLinesPerQuad) {
+        const uint2 m2 = product(__byte_perm(list, 0, 0x4424)), m3 = product(__byte_perm(list, 0, 0x4434));
+        g.x |= m2.x | m3.x, g.y |= m2.y | m3.y;
+        if (list >> 24 != kLinesPerQuad) {
+          const uint32_t* more = cover + (c_tab.yoff[col ? no : nc] + t) * (kCoverBytes / 4);
+          for (int w = 1; w < kCoverBytes / 4; w++) {
+            const uint32_t l4 = __ldg(more + w);
+            if ((l4 & 0xFFu) == kLinesPerQuad) break;
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+              const uint2 m = product(__byte_perm(l4, 0, 0x4404 + 16 * b));
+              g.x |= m.x, g.y |= m.y;
+            }
+          }
+        }
+      }
+      sm.G[col][t][lane] = g;
+    }
+  }
+  __syncthreads();
+  // The moves in the fixed quadrants, in the room of the line products: child
+  // address at Q's state 0, with the turn in the low bits.
+  if (tk.rm >= 0) {
+    uint64_t* moves = reinterpret_cast<uint64_t*>(&sm.M[0][0][0]) + lane;
+    int f = 0;
+#pragma unroll
+    for (int R = 0; R < 4; R++) {
+      if (R == Q) continue;
+      uint64_t base = 0;
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (q != R && q != Q) base += (uint64_t)idx[q] * tk.cstride[R][q];
+      const int empties = 9 - tk.bw[R][0] - tk.bw[R][1];
+      const uint16_t* mv = c_tab.qmoves + ((c - 1) * kMinStates + tk.qoff[R] + idx[R]) * kMoveSlots;
+      for (int i = 0; i < empties; i++, f++) {
+        if (f % kTabWarps != warp) continue;
+        const uint32_t v = __ldg(mv + i);
+        moves[f * 32] =
+            reinterpret_cast<uint64_t>(tk.child[R] + base + (uint64_t)(v & 0xFFFu) * tk.cstride[R][R]) | (v >> 12);
+      }
+    }
+    __syncthreads();
+  }
+  const pp_super* qchild = tk.child[Q];
+#pragma unroll
+  for (int q = 0; q < 4; q++)
+    if (q != Q) qchild += (uint64_t)idx[q] * tk.cstride[Q][q];
+  const uint32_t dq = tk.dim[Q], parts = tk.parts, left = tk.lines - group * 32;
+  const uint32_t s0 = dq * part / parts, s1 = dq * (part + 1) / parts;
+  const int qmoves = 9 - nc - no;
+  switch (tk.rm) {
+    case -1: table_walk<Q, -1>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+    case 0: if constexpr (Q != 0) table_walk<Q, 0>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+    case 1: if constexpr (Q != 1) table_walk<Q, 1>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+    case 2: if constexpr (Q != 2) table_walk<Q, 2>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+    case 3: if constexpr (Q != 3) table_walk<Q, 3>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+    default: table_walk<Q, 4>(tk, sm, warp, s0, s1, qmoves, obase, qchild, left, out); break;
+  }
+}
+
+// Index of the last task whose first block is <= b: 32 probes at a time.
+template <typename T>
+__device__ __forceinline__ int find_block_owner_warp(const T* __restrict__ d, int n, uint32_t b) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0;
+  while (n > 1) {  // the owner is one of d[lo .. lo + n)
+    const int step = (n + 31) / 32, at = lo + lane * step;
+    const bool below = lane * step < n && d[at].block0 <= b;
+    const int last = 31 - __clz(__ballot_sync(0xFFFFFFFFu, below));  // probe 0 always holds
+    n = min(step, n - last * step);
+    lo += last * step;
+  }
+  return lo;
+}
+
+// Every line task of a step: a block finds its task and its 32 lines and range
+// of Q's states within it.
+__global__ void __launch_bounds__(kTabWarps * 32, PP_TAB_MINB)
+    table_line_kernel(const SecLineTask* __restrict__ tasks, int ntasks, pp_super* __restrict__ out) {
+  extern __shared__ uint4 table_smem[];
+  __shared__ SecLineTask tk;
+  TableSmem& sm = *reinterpret_cast<TableSmem*>(table_smem);
+  if (threadIdx.x < 32) {
+    const SecLineTask* src = tasks + find_block_owner_warp(tasks, ntasks, blockIdx.x);
+    static_assert(sizeof(SecLineTask) % 4 == 0, "copied by words");
+    for (int i = threadIdx.x; i < (int)(sizeof(SecLineTask) / 4); i += 32)
+      reinterpret_cast<uint32_t*>(&tk)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+  } else if (threadIdx.x < 96) {
+    const int i = threadIdx.x - 32;
+    sm.K[i / 32][i % 32] = make_uint2(0, 0);
+    sm.M[i / 32][kLinesPerQuad][i % 32] = make_uint2(0, 0);
+  }
+  __syncthreads();
+  const uint32_t b = blockIdx.x - tk.block0, group = b / tk.parts, part = b % tk.parts;
+  switch (tk.q) {
+    case 0: table_lines<0>(tk, group, part, sm, out); break;
+    case 1: table_lines<1>(tk, group, part, sm, out); break;
+    case 2: table_lines<2>(tk, group, part, sm, out); break;
+    default: table_lines<3>(tk, group, part, sm, out); break;
   }
 }
 
@@ -1906,6 +2355,15 @@ int upload_tables(const HostTables& t, DeviceTables* dt, std::string* err) {
   if (!e) e = cudaMemcpy(st, t.standard, sizeof(t.standard), cudaMemcpyHostToDevice);
   if (!e) e = cudaMemcpy(ql, t.qlist, sizeof(t.qlist), cudaMemcpyHostToDevice);
   if (!e) e = cudaMemcpy(fm, t.forms, sizeof(t.forms), cudaMemcpyHostToDevice);
+  void *ls = nullptr, *lc = nullptr, *yr = nullptr, *mv = nullptr;
+  if (!e) e = cudaMalloc(&ls, sizeof(t.lsets));
+  if (!e) e = cudaMemcpy(ls, t.lsets, sizeof(t.lsets), cudaMemcpyHostToDevice);
+  if (!e) e = cudaMalloc(&lc, sizeof(t.lcover));
+  if (!e) e = cudaMemcpy(lc, t.lcover, sizeof(t.lcover), cudaMemcpyHostToDevice);
+  if (!e) e = cudaMalloc(&yr, sizeof(t.yrank));
+  if (!e) e = cudaMemcpy(yr, t.yrank, sizeof(t.yrank), cudaMemcpyHostToDevice);
+  if (!e) e = cudaMalloc(&mv, sizeof(t.qmoves));
+  if (!e) e = cudaMemcpy(mv, t.qmoves, sizeof(t.qmoves), cudaMemcpyHostToDevice);
   if (e) {
     if (err) *err = std::string("table upload: ") + cudaGetErrorString(e);
     return (int)e;
@@ -1918,6 +2376,12 @@ int upload_tables(const HostTables& t, DeviceTables* dt, std::string* err) {
   h.qsorted = (const uint32_t*)qs;
   h.dmin = (const uint16_t*)dmn;
   h.subsets = (const uint16_t*)sub;
+  h.lsets = (const uint32_t*)ls;
+  h.lcover = (const uint32_t*)lc;
+  h.yrank = (const uint32_t*)yr;
+  h.qmoves = (const uint16_t*)mv;
+  std::memcpy(h.ltouch, t.ltouch, sizeof h.ltouch);
+  std::memcpy(h.yoff, t.yoff, sizeof h.yoff);
   for (int b = 0; b < 10; b++)
     for (int w = 0; w < 10; w++) h.qoff[b][w] = t.qoff[b][w], h.qdim[b][w] = t.qdim[b][w];
   e = cudaMemcpyToSymbol(c_tab, &h, sizeof(h));
@@ -2107,51 +2571,55 @@ int launch_line35(const LineTask* d_tasks, int ntasks, uint32_t warps, pp_super*
   return (int)cudaGetLastError();
 }
 
-template <int Q, int RM, bool READY>
-static cudaError_t launch_lines_qrr(unsigned blocks, const SecLineTask* d_tasks, int ntasks, pp_super* d_out,
-                                    pp_stream s) {
+template <int Q, int RM>
+static cudaError_t launch_lines_qr(unsigned blocks, const SecLineTask* d_tasks, int ntasks, pp_super* d_out,
+                                   pp_stream s) {
   // more than the 48 KB of static shared memory: opt in once per instance
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      section_line_kernel<Q, RM, READY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSecLineSmem);
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(section_line_kernel<Q, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSecLineSmem);
   if (attr) return attr;
-  section_line_kernel<Q, RM, READY><<<blocks, kSecLineWarps * 32, kSecLineSmem, s>>>(d_tasks, ntasks, d_out);
+  section_line_kernel<Q, RM><<<blocks, kSecLineWarps * 32, kSecLineSmem, s>>>(d_tasks, ntasks, d_out);
   return cudaSuccess;
 }
 
-template <int Q, int RM>
-static cudaError_t launch_lines_qr(bool ready, unsigned blocks, const SecLineTask* d_tasks, int ntasks,
-                                   pp_super* d_out, pp_stream s) {
-  return ready ? launch_lines_qrr<Q, RM, true>(blocks, d_tasks, ntasks, d_out, s)
-               : launch_lines_qrr<Q, RM, false>(blocks, d_tasks, ntasks, d_out, s);
-}
-
 template <int Q>
-static cudaError_t launch_lines_q(int rm, bool ready, unsigned blocks, const SecLineTask* d_tasks, int ntasks,
+static cudaError_t launch_lines_q(int rm, unsigned blocks, const SecLineTask* d_tasks, int ntasks,
                                   pp_super* d_out, pp_stream s) {
   switch (rm) {
-    case -1: return launch_lines_qr<Q, -1>(ready, blocks, d_tasks, ntasks, d_out, s);
-    case 0: if constexpr (Q != 0) return launch_lines_qr<Q, 0>(ready, blocks, d_tasks, ntasks, d_out, s); break;
-    case 1: if constexpr (Q != 1) return launch_lines_qr<Q, 1>(ready, blocks, d_tasks, ntasks, d_out, s); break;
-    case 2: if constexpr (Q != 2) return launch_lines_qr<Q, 2>(ready, blocks, d_tasks, ntasks, d_out, s); break;
-    case 3: if constexpr (Q != 3) return launch_lines_qr<Q, 3>(ready, blocks, d_tasks, ntasks, d_out, s); break;
-    default: return launch_lines_qr<Q, 4>(ready, blocks, d_tasks, ntasks, d_out, s);
+    case -1: return launch_lines_qr<Q, -1>(blocks, d_tasks, ntasks, d_out, s);
+    case 0: if constexpr (Q != 0) return launch_lines_qr<Q, 0>(blocks, d_tasks, ntasks, d_out, s); break;
+    case 1: if constexpr (Q != 1) return launch_lines_qr<Q, 1>(blocks, d_tasks, ntasks, d_out, s); break;
+    case 2: if constexpr (Q != 2) return launch_lines_qr<Q, 2>(blocks, d_tasks, ntasks, d_out, s); break;
+    case 3: if constexpr (Q != 3) return launch_lines_qr<Q, 3>(blocks, d_tasks, ntasks, d_out, s); break;
+    default: return launch_lines_qr<Q, 4>(blocks, d_tasks, ntasks, d_out, s);
   }
   return cudaErrorInvalidValue;
 }
 
 int launch_section_lines(int q, int rm, const SecLineTask* d_tasks, int ntasks, uint32_t warps, pp_super* d_out,
-                         pp_stream s, bool ready) {
+                         pp_stream s) {
   if (!warps || !ntasks) return 0;
   if (rm == q || rm < -1 || rm > 4) return (int)cudaErrorInvalidValue;
   const unsigned blocks = (warps + kSecLineWarps - 1) / kSecLineWarps;
   cudaError_t e;
   switch (q) {
-    case 0: e = launch_lines_q<0>(rm, ready, blocks, d_tasks, ntasks, d_out, s); break;
-    case 1: e = launch_lines_q<1>(rm, ready, blocks, d_tasks, ntasks, d_out, s); break;
-    case 2: e = launch_lines_q<2>(rm, ready, blocks, d_tasks, ntasks, d_out, s); break;
-    default: e = launch_lines_q<3>(rm, ready, blocks, d_tasks, ntasks, d_out, s); break;
+    case 0: e = launch_lines_q<0>(rm, blocks, d_tasks, ntasks, d_out, s); break;
+    case 1: e = launch_lines_q<1>(rm, blocks, d_tasks, ntasks, d_out, s); break;
+    case 2: e = launch_lines_q<2>(rm, blocks, d_tasks, ntasks, d_out, s); break;
+    default: e = launch_lines_q<3>(rm, blocks, d_tasks, ntasks, d_out, s); break;
   }
   if (e) return (int)e;
+  count_launch();
+  return (int)cudaGetLastError();
+}
+
+int launch_table_lines(const SecLineTask* d_tasks, int ntasks, uint32_t blocks, pp_super* d_out, pp_stream s) {
+  if (!blocks || !ntasks) return 0;
+  // more than the 48 KB of static shared memory: opt in once
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(table_line_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TableSmem));
+  if (attr) return (int)attr;
+  table_line_kernel<<<blocks, kTabWarps * 32, sizeof(TableSmem), s>>>(d_tasks, ntasks, d_out);
   count_launch();
   return (int)cudaGetLastError();
 }

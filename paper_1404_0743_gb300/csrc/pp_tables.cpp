@@ -187,8 +187,50 @@ void build(HostTables& t) {
         if (__builtin_popcount(v) <= c) t.subsets[at++] = (uint16_t)v;
     if (at != kCappedSubsets) std::abort();
   }
-  // five-in-a-row forms
   std::vector<LineInfo> lines = all_lines();
+  // pattern tables of the line kernels
+  if (lines.size() != 32) std::abort();
+  for (int q = 0; q < 4; q++) {
+    for (int l = 0; l < 32; l++)
+      if (lines[l].part[q]) t.ltouch[q] |= 1u << l;
+    if (__builtin_popcount(t.ltouch[q]) != kLinesPerQuad) std::abort();
+    for (uint32_t x = 0; x < 512; x++)
+      for (int l = 0; l < 32; l++)
+        t.lsets[q][x][l / 8] |= cover_set(lines[l].part[q], x) << (4 * (l % 8));  // 0xF for an empty part
+  }
+  uint8_t place[512];
+  for (int n = 0, at = 0; n <= 10; n++) {
+    t.yoff[n] = (uint16_t)at;
+    for (uint32_t x = 0; x < 512; x++) {
+      if (__builtin_popcount(x) != n) continue;
+      place[x] = (uint8_t)(at - t.yoff[n]);
+      for (int q = 0; q < 4; q++) {
+        int slot = 0, listed = 0;
+        std::memset(t.lcover[q][at], kLinesPerQuad, kCoverBytes);
+        for (int l = 0; l < 32; l++) {
+          const uint32_t part = lines[l].part[q];
+          if (!part) continue;
+          if ((x & part) == part) t.lcover[q][at][listed++] = (uint8_t)slot;
+          slot++;
+        }
+      }
+      at++;
+    }
+  }
+  for (int i = 0; i < kMinStates; i++)
+    for (int c = 0; c < 2; c++) {
+      const int code = t.qlist[i];
+      const uint32_t d = t.qdecode[code];
+      uint32_t x = d >> (9 * c) & 0x1FFu;
+      for (int turn = 0; turn < 4; turn++, x = rotate9(x)) t.yrank[i][c] |= (uint32_t)place[x] << (8 * turn);
+      int at = 0;
+      for (int e = 0; e < 9; e++) {
+        if ((d | d >> 9) >> e & 1) continue;
+        const uint32_t st = t.standard[code + (c + 1) * pow3i(e)];
+        t.qmoves[c][i][at++] = (uint16_t)((st & 0xFFFu) | (st >> 16) << 12);
+      }
+    }
+  // five-in-a-row forms
   auto group = [&](int quads) {
     std::vector<LineInfo> g;
     for (auto& l : lines)
