@@ -340,7 +340,7 @@ int pp_quadrant_states(int black, int white, uint16_t* codes, int max) {
 
 int pp_slice_sections(int n, pp_section_desc* out, int max, uint64_t* total) {
   if (n < 0 || n > 36) return -fail(PP_EINVAL, "slice %d out of range", n);
-  auto secs = slice_sections(n, total);
+  const auto& secs = slice_sections(n, total);
   if (out)
     for (size_t i = 0; i < secs.size() && (int)i < max; i++) out[i] = secs[i];
   return (int)secs.size();
@@ -777,8 +777,8 @@ int build_tasks(int n, const std::vector<pp_section_desc>& secs, const std::vect
                 std::vector<SecTask>* tasks, uint32_t* blocks, bool d4 = false,
                 const uint64_t* in_offsets = nullptr, uint64_t in_count = 0) {
   const HostTables& t = host_tables();
-  std::vector<pp_section_desc> next;
-  if (n < 36 && !child_ptrs) next = d4 ? slice_sections_d4(n + 1, nullptr) : slice_sections(n + 1, nullptr);
+  static const std::vector<pp_section_desc> none;
+  const auto& next = n == 36 || child_ptrs ? none : d4 ? slice_sections_d4(n + 1, nullptr) : slice_sections(n + 1, nullptr);
   const int mover = (n % 2 == 0) ? 1 : 2;
   uint64_t start = 0, nblocks = 0;
   for (int si : which) {
@@ -885,7 +885,7 @@ int build_line35(const std::vector<pp_section_desc>& secs, const std::vector<int
                  bool d4 = false) {
   const HostTables& t = host_tables();
   uint64_t total36 = 0;
-  std::vector<pp_section_desc> next = d4 ? slice_sections_d4(36, &total36) : slice_sections(36, &total36);
+  const auto& next = d4 ? slice_sections_d4(36, &total36) : slice_sections(36, &total36);
   std::vector<LineTask> tasks;
   uint64_t start = 0;
   W->on_demand = !child_ptrs && !in_values;
@@ -1338,7 +1338,7 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
   }
   const HostTables& t = host_tables();
   uint64_t total = 0;
-  auto secs = d4 ? slice_sections_d4(n + 1, &total) : slice_sections(n + 1, &total);
+  const auto& secs = d4 ? slice_sections_d4(n + 1, &total) : slice_sections(n + 1, &total);
   std::vector<LineTask> tasks;
   std::vector<std::pair<uint64_t, uint64_t>> spans;  // [first, end) of every section held
   for (size_t i = 0; i < secs.size(); i++) {
@@ -1421,7 +1421,7 @@ int slice_step(int n, const pp_super* in_values, pp_super* out_values, const uin
   if (n < 36 && !on_demand && (!in_values || !aligned32(in_values)))
     return fail(PP_EINVAL, "slice %d needs slice %d values (32-byte aligned)", n, n + 1);
   if (!out_values || !aligned32(out_values)) return fail(PP_EINVAL, "output must be non-null and 32-byte aligned");
-  auto secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
+  const auto& secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
   std::vector<int> which;
   for (size_t i = 0; i < secs.size(); i++)
     if (!filter || filter[i]) which.push_back((int)i);
@@ -1532,8 +1532,8 @@ int pp_slice_step_sparse(int n, int d4, const pp_super* in_values, const uint64_
 int pp_slice_children(int n, int d4, const uint8_t* filter, uint8_t* child_filter) {
   if (n < 0 || n > 35) return fail(PP_EINVAL, "slice %d has no child slice", n);
   if (!child_filter) return fail(PP_EINVAL, "null child filter");
-  auto secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
-  auto next = d4 ? slice_sections_d4(n + 1, nullptr) : slice_sections(n + 1, nullptr);
+  const auto& secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
+  const auto& next = d4 ? slice_sections_d4(n + 1, nullptr) : slice_sections(n + 1, nullptr);
   std::memset(child_filter, 0, next.size());
   const int mover = (n % 2 == 0) ? 1 : 2;
   for (size_t i = 0; i < secs.size(); i++) {
@@ -1558,7 +1558,7 @@ int pp_slice_children(int n, int d4, const uint8_t* filter, uint8_t* child_filte
 
 int pp_d4_slice_sections(int n, pp_section_desc* out, int max, uint64_t* total) {
   if (n < 0 || n > 36) return -fail(PP_EINVAL, "slice %d out of range", n);
-  auto secs = slice_sections_d4(n, total);
+  const auto& secs = slice_sections_d4(n, total);
   for (int i = 0; out && i < max && i < (int)secs.size(); i++) out[i] = secs[i];
   return (int)secs.size();
 }
@@ -1641,7 +1641,7 @@ int slice_plan_create(int n, const pp_super* in_values, pp_super* out_values, co
   P->d4 = d4;
   P->out = out_values;
   P->line = (n == 35 || n == 36) && stage != 2;
-  auto secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
+  const auto& secs = d4 ? slice_sections_d4(n, nullptr) : slice_sections(n, nullptr);
   std::vector<int> which;
   for (size_t i = 0; i < secs.size(); i++)
     if (!filter || filter[i]) which.push_back((int)i);

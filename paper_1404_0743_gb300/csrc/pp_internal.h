@@ -112,8 +112,9 @@ struct HostTables {
 const HostTables& host_tables();
 uint32_t rotate9(uint32_t mask);  // one anticlockwise turn of a 9-bit pattern
 
-// Sections of slice n (count tuples in increasing order), offsets back to back.
-std::vector<pp_section_desc> slice_sections(int n, uint64_t* total);
+// Sections of slice n, 0 <= n <= 36 (count tuples in increasing order), offsets
+// back to back; enumerated at the first call.
+const std::vector<pp_section_desc>& slice_sections(int n, uint64_t* total);
 int section_index(const std::vector<pp_section_desc>& secs, const uint8_t bw[4][2]);
 
 // ---------------------------------------------------------------------------
@@ -143,7 +144,7 @@ PP_HD constexpr bool sym_reflects(int s) { return (s >> 2) != 0; }
 // D4-minimal sections of slice n (paper, "Data layout and distribution": a
 // section is computed only when its count tuple is the least of its eight
 // images), in increasing order, offsets back to back.
-std::vector<pp_section_desc> slice_sections_d4(int n, uint64_t* total);
+const std::vector<pp_section_desc>& slice_sections_d4(int n, uint64_t* total);
 // Quadrant code under symmetry s's local action (mirror, then s & 3 turns).
 int symmetry_pattern(int s, int code);
 // The least image of a count tuple and the first symmetry reaching it.

@@ -295,7 +295,17 @@ const HostTables& host_tables() {
   return *t;
 }
 
-std::vector<pp_section_desc> slice_sections(int n, uint64_t* total) {
+namespace {
+
+// The lists are constants of the layout: each is enumerated once (0.2-2 ms)
+// and kept for the life of the process (at most 16,361 sections a slice).
+struct SectionList {
+  std::once_flag once;
+  std::vector<pp_section_desc> secs;
+  uint64_t total = 0;
+};
+
+std::vector<pp_section_desc> enumerate_sections(int n, uint64_t* total) {
   const HostTables& t = host_tables();
   std::vector<pp_section_desc> out;
   const int B = (n + 1) / 2, W = n / 2;
@@ -321,8 +331,18 @@ std::vector<pp_section_desc> slice_sections(int n, uint64_t* total) {
         offset += size;
         out.push_back(d);
       }
-  if (total) *total = offset;
+  *total = offset;
   return out;
+}
+
+}  // namespace
+
+const std::vector<pp_section_desc>& slice_sections(int n, uint64_t* total) {
+  static SectionList lists[37];
+  SectionList& L = lists[n];
+  std::call_once(L.once, [&] { L.secs = enumerate_sections(n, &L.total); });
+  if (total) *total = L.total;
+  return L.secs;
 }
 
 int least_image(const uint8_t bw[4][2], uint8_t out[4][2]) {
@@ -341,19 +361,21 @@ int least_image(const uint8_t bw[4][2], uint8_t out[4][2]) {
   return best_s;
 }
 
-std::vector<pp_section_desc> slice_sections_d4(int n, uint64_t* total) {
-  std::vector<pp_section_desc> out;
-  uint64_t offset = 0;
-  for (pp_section_desc d : slice_sections(n, nullptr)) {
-    uint8_t least[4][2];
-    least_image(d.bw, least);
-    if (std::memcmp(least, d.bw, sizeof least) != 0) continue;
-    d.offset = offset;
-    offset += (uint64_t)d.dim[0] * d.dim[1] * d.dim[2] * d.dim[3];
-    out.push_back(d);
-  }
-  if (total) *total = offset;
-  return out;
+const std::vector<pp_section_desc>& slice_sections_d4(int n, uint64_t* total) {
+  static SectionList lists[37];
+  SectionList& L = lists[n];
+  std::call_once(L.once, [&] {
+    for (pp_section_desc d : slice_sections(n, nullptr)) {
+      uint8_t least[4][2];
+      least_image(d.bw, least);
+      if (std::memcmp(least, d.bw, sizeof least) != 0) continue;
+      d.offset = L.total;
+      L.total += (uint64_t)d.dim[0] * d.dim[1] * d.dim[2] * d.dim[3];
+      L.secs.push_back(d);
+    }
+  });
+  if (total) *total = L.total;
+  return L.secs;
 }
 
 int section_index(const std::vector<pp_section_desc>& secs, const uint8_t bw[4][2]) {
