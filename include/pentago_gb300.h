@@ -136,7 +136,9 @@ typedef struct pp_batch_opts {
  * masks instead of evaluating lines), then room for n results used by
  * pp_midgame_solve_host: at most
  * n (F(max_empty) 64 + 2^max_empty 64 + 64) bytes, as
- * pp_midgame_workspace_bytes gives.
+ * pp_midgame_workspace_bytes gives.  Boards that share their number of empty
+ * cells (7 or more) are solved sixteen at a time, their tables interleaved
+ * over the room of the sixteen; the others one by one.
  */
 int pp_midgame_workspace_bytes(int n, int max_empty, size_t* bytes);
 

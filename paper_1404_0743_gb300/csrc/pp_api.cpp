@@ -16,6 +16,7 @@
 #include <memory>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "pp_internal.h"
@@ -135,7 +136,16 @@ int describe_board(uint64_t packed, int max_empty, MidBoard* mb, int i) {
   return PP_OK;
 }
 
-std::map<std::pair<int, int>, std::unique_ptr<LevelLists>> g_lists;
+// Fewest empty cells solved in packs: from 7 on sixteen boards of one shape
+// take no longer in a pack than one by one (16 boards with 7 empty cells: 55
+// against 57 us, with 12: 145 against 179), below it a few per cent more (16
+// with 5: 41 against 38; the launch is latency there).
+#ifndef PP_PACK_MIN_EMPTY
+#define PP_PACK_MIN_EMPTY 7
+#endif
+constexpr int kPackMinEmpty = PP_PACK_MIN_EMPTY;
+
+std::map<std::tuple<int, int, bool>, std::unique_ptr<LevelLists>> g_lists;
 
 }  // namespace
 
@@ -166,7 +176,7 @@ uint64_t fills_total(int k) {
   return table[k];
 }
 
-void build_fill_lists(int k, int mover, FillLists* L) {
+void build_fill_lists(int k, int mover, bool grouped, FillLists* L) {
   std::vector<std::vector<uint64_t>> per(k + 1);
   const uint64_t total = pow3u(k);
   const int other = 3 - mover;
@@ -195,14 +205,23 @@ void build_fill_lists(int k, int mover, FillLists* L) {
   uint64_t p3[17];
   p3[0] = 1;
   for (int i = 1; i <= 16; i++) p3[i] = p3[i - 1] * 3;
+  std::vector<uint32_t> at;  // per stone set of the colour not to move: its next place in the level's list
   for (int m = 0; m <= k; m++) {
+    const uint64_t c = (m & 1) ? (uint64_t)other : (uint64_t)mover;  // colour placed at level m
+    std::vector<uint64_t> level = per[m];
+    if (grouped) {  // by the stones of the colour that does not move (a counting sort)
+      auto still = [&](uint64_t e) { return (uint32_t)(c == 1 ? e >> 48 : e >> 32 & 0xFFFFu); };
+      at.assign(((size_t)1 << k) + 1, 0);
+      for (uint64_t e : per[m]) at[still(e) + 1]++;
+      for (size_t i = 1; i < at.size(); i++) at[i] += at[i - 1];
+      for (uint64_t e : per[m]) level[at[still(e)]++] = e;
+    }
     L->offset.push_back(L->flat.size());
-    L->count.push_back((uint32_t)per[m].size());
-    L->flat.insert(L->flat.end(), per[m].begin(), per[m].end());
+    L->count.push_back((uint32_t)level.size());
+    for (uint64_t e : level) L->flat.push_back((e & ~(uint64_t)0xFFFFFFFFu) | pos[e & 0xFFFFFFFFu]);
     L->ranks_at.push_back(L->ranks.size());
     if (m == k) continue;
-    const uint64_t c = (m & 1) ? (uint64_t)other : (uint64_t)mover;  // colour placed at level m
-    for (uint64_t e : per[m]) {
+    for (uint64_t e : level) {
       const uint64_t idx = e & 0xFFFFFFFFu;
       const uint32_t filled = (uint32_t)(e >> 32 & 0xFFFFu) | (uint32_t)(e >> 48);
       for (int i = 0; i < k; i++)
@@ -211,15 +230,15 @@ void build_fill_lists(int k, int mover, FillLists* L) {
   }
 }
 
-const LevelLists* level_lists(int k, int mover, std::string* err) {
-  auto key = std::make_pair(k, mover);
+const LevelLists* level_lists(int k, int mover, std::string* err, bool grouped) {
+  auto key = std::make_tuple(k, mover, grouped);
   auto it = g_lists.find(key);
   if (it != g_lists.end()) return it->second.get();
   auto L = std::make_unique<LevelLists>();
   L->k = k;
   L->mover = mover;
   FillLists F;
-  build_fill_lists(k, mover, &F);
+  build_fill_lists(k, mover, grouped, &F);
   L->offset = F.offset;
   L->count = F.count;
   L->ranks_at = F.ranks_at;
@@ -251,10 +270,14 @@ struct pp_midgame_plan {
   int n = 0, max_empty = 0, kmax = 0;
   uint64_t table_entries = 0;  // compact fill-table entries of all boards
   void* d_mem = nullptr;  // one allocation holding the four arrays below
-  MidBoard* d_boards = nullptr;
+  MidBoard* d_boards = nullptr;  // the packs' boards, then the others
   MidSeg* d_segs = nullptr;
   using Level = MidLevel;
-  std::vector<Level> levels;  // levels[j] is stones added m = kmax - j
+  // packs of boards of one shape, and the boards left over one by one: each
+  // with its own levels, levels[j] being stones added m = kmax - j
+  int npacks = 0, pack_kmax = 0;
+  std::vector<Level> pack_levels, levels;
+  MidLevel* d_pack_levels = nullptr;
   MidLevel* d_levels = nullptr;
   uint32_t* d_sync = nullptr;  // barrier count, generation, status (persistent mode)
   int mode = 1;                // 1 persistent, 2 one launch per level, 3 graph of level launches
@@ -385,86 +408,111 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
   for (int i = 0; i < n; i++) {
     int rc = describe_board(h_boards[i], max_empty, &boards[i], i);
     if (rc) return rc;
-    boards[i].table = P->table_entries;  // boards' compact tables back to back
-    P->table_entries += fills_total((int)boards[i].k);
     boards[i].out = (uint64_t)i;
-    boards[i].masks = (uint64_t)i * mask_entries_per_board(max_empty);
-    P->kmax = std::max(P->kmax, (int)boards[i].k);
   }
+  int per_k[kMaxEmpty + 1] = {};
+  for (const MidBoard& b : boards) per_k[b.k]++;
   {
-    int per_k[kMaxEmpty + 1] = {};
-    for (const MidBoard& b : boards) per_k[b.k]++;
     P->shape = "max_empty=" + std::to_string(max_empty) + " boards=";
     for (int k = 0; k <= kMaxEmpty; k++)
       if (per_k[k]) P->shape += std::to_string(k) + ":" + std::to_string(per_k[k]) + ",";
   }
+  // whole packs of one shape first (the number of empty cells decides the
+  // mover), then the other boards in their given order
+  {
+    int taken[kMaxEmpty + 1] = {}, in_packs[kMaxEmpty + 1], first[kMaxEmpty + 1];
+    int at = 0;
+    for (int k = kMaxEmpty; k >= 0; k--) {
+      in_packs[k] = k >= kPackMinEmpty ? per_k[k] / kPackBoards * kPackBoards : 0;
+      first[k] = at;
+      at += in_packs[k];
+      if (in_packs[k]) P->pack_kmax = std::max(P->pack_kmax, k);
+    }
+    P->npacks = at / kPackBoards;
+    std::vector<MidBoard> sorted(n);
+    for (const MidBoard& b : boards) {
+      const int k = (int)b.k;
+      sorted[taken[k] < in_packs[k] ? first[k] + taken[k] : at++] = b;
+      taken[k]++;
+    }
+    boards = std::move(sorted);
+  }
+  for (int i = 0; i < n; i++) {
+    boards[i].table = P->table_entries;  // boards' compact tables back to back
+    P->table_entries += fills_total((int)boards[i].k);
+    boards[i].masks = (uint64_t)i * mask_entries_per_board(max_empty);
+    if (i >= P->npacks * kPackBoards) P->kmax = std::max(P->kmax, (int)boards[i].k);
+  }
   std::vector<MidSeg> segs;
   {
     std::lock_guard<std::mutex> lock(g_mutex);
-    // each board's level lists, looked up once per (empty cells, mover)
-    std::vector<const LevelLists*> lists(n);
-    const LevelLists* memo[kMaxEmpty + 1][3] = {};
-    for (int i = 0; i < n; i++) {
-      const LevelLists*& L = memo[boards[i].k][boards[i].mover];
-      if (!L) {
+    // One level's descriptors: units are packs (their first boards) or single
+    // boards, `per_block` fills to a block.  When all are of one shape a
+    // level has one shared descriptor, unit j being the j-th.
+    auto add_levels = [&](int first, int units, int stride, uint32_t per_block, bool grouped, int kmax,
+                          std::vector<pp_midgame_plan::Level>* levels) {
+      const LevelLists* memo[kMaxEmpty + 1][3] = {};
+      bool same = true;
+      for (int u = 0; u < units; u++) {
+        const MidBoard& b = boards[first + u * stride];
+        const LevelLists*& L = memo[b.k][b.mover];
         std::string err;
-        if (!(L = level_lists((int)boards[i].k, (int)boards[i].mover, &err))) return fail(PP_ECUDA, "%s", err.c_str());
+        if (!L && !(L = level_lists((int)b.k, (int)b.mover, &err, grouped))) return fail(PP_ECUDA, "%s", err.c_str());
+        same = same && b.k == boards[first].k && b.mover == boards[first].mover;
       }
-      lists[i] = L;
-    }
-    bool same = n > 0;  // every board with the same empty cells and mover
-    for (int i = 1; i < n && same; i++) same = boards[i].k == boards[0].k && boards[i].mover == boards[0].mover;
-    if (!same) segs.reserve((size_t)n * (P->kmax + 1));
-    for (int m = P->kmax; m >= 0 && same; m--) {
-      // one shared descriptor per level: segment j is board j
-      const LevelLists* L = lists[0];
-      MidSeg s{};
-      s.list = L->d_entries + L->offset[m];
-      s.ranks = L->d_ranks + L->ranks_at[m];
-      s.loff = (uint32_t)L->offset[m];
-      s.coff = m < P->kmax ? (uint32_t)L->offset[m + 1] : 0u;
-      s.count = L->count[m];
-      s.level = (uint32_t)m;
-      const uint32_t per = (s.count + kBlock - 1) / kBlock;
-      if ((uint64_t)per * (uint64_t)n >= (1ull << 31)) return fail(PP_EINVAL, "too many boards for one level launch");
-      pp_midgame_plan::Level lv{(int)segs.size(), n, per * (uint32_t)n, per | kSharedSegs};
-      segs.push_back(s);
-      P->levels.push_back(lv);
-    }
-    for (int m = P->kmax; m >= 0 && n > 0 && !same; m--) {
-      pp_midgame_plan::Level lv{(int)segs.size(), 0, 0, 0};
-      for (int i = 0; i < n; i++) {
-        if ((int)boards[i].k < m) continue;
-        const LevelLists* L = lists[i];
-        MidSeg s{};
-        s.block0 = lv.blocks;
-        s.list = L->d_entries + L->offset[m];
-        s.ranks = L->d_ranks + L->ranks_at[m];
-        s.loff = (uint32_t)L->offset[m];
-        s.coff = m < (int)boards[i].k ? (uint32_t)L->offset[m + 1] : 0u;
-        s.count = L->count[m];
-        s.board = (uint32_t)i;
-        s.level = (uint32_t)m;
-        lv.blocks += (s.count + kBlock - 1) / kBlock;
-        segs.push_back(s);
-        lv.nsegs++;
+      if (!same) segs.reserve(segs.size() + (size_t)units * (kmax + 1));
+      for (int m = kmax; m >= 0 && units > 0; m--) {
+        pp_midgame_plan::Level lv{(int)segs.size(), 0, 0, 0};
+        uint64_t blocks = 0;
+        for (int u = 0; u < (same ? 1 : units); u++) {
+          const MidBoard& b = boards[first + u * stride];
+          if ((int)b.k < m) continue;
+          const LevelLists* L = memo[b.k][b.mover];
+          MidSeg s{};
+          s.block0 = (uint32_t)blocks;
+          s.list = L->d_entries + L->offset[m];
+          s.ranks = L->d_ranks + L->ranks_at[m];
+          s.loff = (uint32_t)L->offset[m];
+          s.coff = m < (int)b.k ? (uint32_t)L->offset[m + 1] : 0u;
+          s.count = L->count[m];
+          s.board = (uint32_t)(first + u * stride);
+          s.level = (uint32_t)m;
+          blocks += (s.count + per_block - 1) / per_block;
+          segs.push_back(s);
+          lv.nsegs++;
+        }
+        if (same) {
+          lv.seg_blocks = (uint32_t)blocks | kSharedSegs;
+          lv.nsegs = units;
+          blocks *= (uint64_t)units;
+        } else {
+          lv.seg_blocks = uniform_seg_blocks(segs.data() + lv.seg0, lv.nsegs, per_block);
+        }
+        if (blocks >= (1ull << 31)) return fail(PP_EINVAL, "too many boards for one level launch");
+        lv.blocks = (uint32_t)blocks;
+        levels->push_back(lv);
       }
-      lv.seg_blocks = uniform_seg_blocks(segs.data() + lv.seg0, lv.nsegs, kBlock);
-      if ((uint64_t)lv.blocks >= (1ull << 31)) return fail(PP_EINVAL, "too many boards for one level launch");
-      P->levels.push_back(lv);
-    }
+      return (int)PP_OK;
+    };
+    const int packed = P->npacks * kPackBoards;
+    int rc = add_levels(0, P->npacks, kPackBoards, kPackFills, true, P->pack_kmax, &P->pack_levels);
+    if (!rc) rc = add_levels(packed, n - packed, 1, kBlock, false, P->kmax, &P->levels);
+    if (rc) return rc;
   }
   if (n > 0) {
     // boards, segments, levels and the barrier words (zero) packed into one
     // allocation and one copy
     auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
     const size_t ob = 0, os = ob + up(boards.size() * sizeof(MidBoard));
-    const size_t ol = os + up(segs.size() * sizeof(MidSeg));
+    const size_t op = os + up(segs.size() * sizeof(MidSeg));
+    const size_t ol = op + up(P->pack_levels.size() * sizeof(MidLevel));
     const size_t oy = ol + up(P->levels.size() * sizeof(MidLevel)), total = oy + 4 * sizeof(uint32_t);
     std::vector<char> pack(total, 0);
     std::memcpy(pack.data() + ob, boards.data(), boards.size() * sizeof(MidBoard));
     std::memcpy(pack.data() + os, segs.data(), segs.size() * sizeof(MidSeg));
-    std::memcpy(pack.data() + ol, P->levels.data(), P->levels.size() * sizeof(MidLevel));
+    if (!P->pack_levels.empty())
+      std::memcpy(pack.data() + op, P->pack_levels.data(), P->pack_levels.size() * sizeof(MidLevel));
+    if (!P->levels.empty()) std::memcpy(pack.data() + ol, P->levels.data(), P->levels.size() * sizeof(MidLevel));
     cudaError_t e;
     if (pooled) {
       // stream-ordered: no device-wide synchronisation; the pageable source
@@ -486,6 +534,7 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     char* base = static_cast<char*>(P->d_mem);
     P->d_boards = reinterpret_cast<MidBoard*>(base + ob);
     P->d_segs = reinterpret_cast<MidSeg*>(base + os);
+    P->d_pack_levels = reinterpret_cast<MidLevel*>(base + op);
     P->d_levels = reinterpret_cast<MidLevel*>(base + ol);
     P->d_sync = reinterpret_cast<uint32_t*>(base + oy);
   }
@@ -495,6 +544,40 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
 
 }  // namespace
 }  // namespace pp
+
+namespace {
+
+int launch_masks(const pp_midgame_plan* P, void* masks, pp_stream s) {
+  const int packed = P->npacks * kPackBoards;
+  int rc = launch_five_tables_packs(P->d_boards, P->npacks, P->pack_kmax, masks, s);
+  if (!rc) rc = launch_five_tables(P->d_boards + packed, P->n - packed, P->kmax, masks, s);
+  return rc;
+}
+
+// One launch per level: the packs' levels, then the other boards'.
+int launch_levels(const pp_midgame_plan* P, void* d_workspace, void* masks, pp_super* d_out, pp_stream s) {
+  int rc = launch_masks(P, masks, s);
+  for (const bool packs : {true, false}) {
+    const auto& levels = packs ? P->pack_levels : P->levels;
+    for (size_t j = 0; !rc && j < levels.size(); j++) {
+      const auto& lv = levels[j];
+      const int last = j + 1 == levels.size() ? 1 : 0;
+      rc = packs ? launch_pack_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
+                                     d_out, last, s, masks, lv.seg_blocks, P->parity)
+                 : launch_midgame_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
+                                        d_out, last, s, masks, lv.seg_blocks, P->parity);
+    }
+  }
+  return rc;
+}
+
+// Kernels of launch_levels: masks and levels of either kind, and the packs'
+// root values.
+uint64_t level_launches(const pp_midgame_plan* P) {
+  return (P->npacks ? P->pack_levels.size() + 2 : 0) + (P->levels.empty() ? 0 : P->levels.size() + 1);
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -509,13 +592,18 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
   // workspace: fill tables of all boards, then their five tables
   void* masks = (char*)d_workspace + (size_t)P->table_entries * fill_entry_bytes(P->parity);
   if (P->mode == 1) {
-    int grid = persistent_midgame_blocks(P->ctas_per_sm, P->parity >= 0);
     cudaError_t e = cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s);
     if (e) return cuda_fail(e, "barrier reset");
-    int rc = launch_five_tables(P->d_boards, P->n, P->kmax, masks, s);
-    if (!rc)
+    int rc = launch_masks(P, masks, s);
+    const bool half = P->parity >= 0;
+    if (!rc && P->npacks)
+      rc = launch_pack_persistent(P->d_boards, P->d_segs, P->d_pack_levels, (int)P->pack_levels.size(), P->d_levels,
+                                  (int)P->levels.size(), (pp_super*)d_workspace, d_out, P->d_sync,
+                                  persistent_pack_blocks(P->ctas_per_sm, half, !P->levels.empty()), s, masks, P->parity);
+    else if (!rc)
       rc = launch_midgame_persistent(P->d_boards, P->d_segs, P->d_levels, (int)P->levels.size(),
-                                     (pp_super*)d_workspace, d_out, P->d_sync, grid, s, masks, P->parity);
+                                     (pp_super*)d_workspace, d_out, P->d_sync,
+                                     persistent_midgame_blocks(P->ctas_per_sm, half), s, masks, P->parity);
     return rc ? cuda_fail(rc, "persistent midgame launch") : PP_OK;
   }
   if (P->mode == 3) {
@@ -529,13 +617,7 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
       e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
       int rc = 0;
       set_launch_counting(false);
-      if (!e) rc = launch_five_tables(P->d_boards, P->n, P->kmax, masks, (pp_stream)cs);
-      for (size_t j = 0; !e && !rc && j < P->levels.size(); j++) {
-        const auto& lv = P->levels[j];
-        rc = launch_midgame_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
-                                  d_out, j + 1 == P->levels.size() ? 1 : 0, (pp_stream)cs, masks, lv.seg_blocks,
-                                  P->parity);
-      }
+      if (!e) rc = launch_levels(P, d_workspace, masks, d_out, (pp_stream)cs);
       set_launch_counting(true);
       cudaError_t e2 = e ? e : cudaStreamEndCapture(cs, &g);
       if (!e2 && !rc) e2 = cudaGraphInstantiate(&P->graph, g, 0);
@@ -547,19 +629,11 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
       P->graph_out = d_out;
     }
     cudaError_t e = cudaGraphLaunch(P->graph, s);
-    add_launches(P->levels.size() + 1);
+    add_launches(level_launches(P));
     return e ? cuda_fail(e, "graph launch") : PP_OK;
   }
-  int e = launch_five_tables(P->d_boards, P->n, P->kmax, masks, s);
-  if (e) return cuda_fail(e, "five tables launch");
-  for (size_t j = 0; j < P->levels.size(); j++) {
-    const auto& lv = P->levels[j];
-    const bool final_level = j + 1 == P->levels.size();
-    e = launch_midgame_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
-                             d_out, final_level ? 1 : 0, s, masks, lv.seg_blocks, P->parity);
-    if (e) return cuda_fail(e, "midgame level launch");
-  }
-  return PP_OK;
+  int e = launch_levels(P, d_workspace, masks, d_out, s);
+  return e ? cuda_fail(e, "midgame level launch") : PP_OK;
 }
 
 int pp_midgame_plan_configure(pp_midgame_plan* P, const pp_batch_opts* opts) {

@@ -187,7 +187,7 @@ struct MidBoard {
 };
 
 // One (board, level) piece of a level launch.  Entries of the level list
-// are (fill index | black slots << 32 | white slots << 48).
+// are (position in the level | black slots << 32 | white slots << 48).
 struct MidSeg {
   uint32_t block0;         // first thread block of this segment (segments start on block boundaries)
   uint32_t loff;           // this level's first entry in the board's compact fill table
@@ -214,9 +214,21 @@ struct MidLevel {
 // derives the rest from the block index.
 constexpr uint32_t kSharedSegs = 0x80000000u;
 
+// Boards of one shape solved together, their tables sliced across them
+// (pack_level_kernel).  A pack's boards have consecutive descriptors; its
+// records and masks take the room of the boards' own, from the first's.  A
+// segment of a pack level names the first board and counts fills, kPackFills
+// to a block.
+constexpr int kPackBoards = 16;
+#ifndef PP_PACK_THREADS
+#define PP_PACK_THREADS 256
+#endif
+constexpr int kPackThreads = PP_PACK_THREADS;  // threads per block, eight to a fill
+constexpr uint32_t kPackFills = kPackThreads / 8;
+
 // Blocks of every segment of a level when all are equal (segment j then
 // starts at block j * that), else 0.
-inline uint32_t uniform_seg_blocks(const MidSeg* segs, int nsegs, uint32_t kblock) {
+inline uint32_t uniform_seg_blocks(const MidSeg* segs, int nsegs, uint32_t kblock) {  // kblock: fills per block
   if (nsegs <= 0) return 0;
   const uint32_t b = (segs[0].count + kblock - 1) / kblock;
   for (int j = 0; j < nsegs; j++)
@@ -224,22 +236,24 @@ inline uint32_t uniform_seg_blocks(const MidSeg* segs, int nsegs, uint32_t kbloc
   return b;
 }
 
-// Level lists for one (k, root mover): for level m, fills with m stones,
-// ceil(m/2) of the root mover's colour; sorted by fill index.
-// Level lists of one (k, root mover), built on the host: level m's fills in
-// increasing fill index, flat, level after level (offset[m] = fills of the
-// levels below m).  A board's compact fill table uses the same positions:
-// the value of fill e of level m sits at offset[m] + e.  For each fill of
-// level m < k and each of its empty slots in increasing order, ranks holds
-// the child's position in level m + 1 (ranks_at[m] + e (k - m) + j).
+// Level lists of one (k, root mover), built on the host, flat, level after
+// level (offset[m] = fills of the levels below m): the fills with m stones,
+// ceil(m/2) of the root mover's colour.  A board's compact fill table keeps a
+// level's fills in increasing fill index: the value of the fill of level m
+// with position pos sits at offset[m] + pos.  The lists are in that order
+// too, or (grouped, for packs) by the slots of the colour not to move, then
+// by fill index: a move leaves those stones, so a group's fills share their
+// children.  For the e-th fill listed of level m < k and each of its empty
+// slots in increasing order, ranks holds the child's position in level m + 1
+// (ranks_at[m] + e (k - m) + j).
 struct FillLists {
-  std::vector<uint64_t> flat;       // idx | black slots << 32 | white slots << 48
+  std::vector<uint64_t> flat;       // pos | black slots << 32 | white slots << 48
   std::vector<uint64_t> offset;     // per level
   std::vector<uint32_t> count;      // per level
   std::vector<uint32_t> ranks;      // child positions
   std::vector<uint64_t> ranks_at;   // per level
 };
-void build_fill_lists(int k, int mover, FillLists* out);
+void build_fill_lists(int k, int mover, bool grouped, FillLists* out);
 uint64_t fills_total(int k);  // fills of every level: sum_m C(k, m) C(m, ceil(m/2))
 
 struct LevelLists {
@@ -251,7 +265,7 @@ struct LevelLists {
   std::vector<uint64_t> ranks_at;  // per level
   uint64_t total = 0;              // entries of a board's compact table
 };
-const LevelLists* level_lists(int k, int mover, std::string* err);
+const LevelLists* level_lists(int k, int mover, std::string* err, bool grouped = false);
 // Host validation of one midgame root (fills everything but table/out).
 int validate_midgame_board(uint64_t packed, int max_empty, MidBoard* mb, int i);
 int report_error(int code, const char* message);  // sets pp_last_error_string
@@ -354,6 +368,8 @@ int launch_midgame_level(const MidBoard* d_boards, const MidSeg* d_segs, int nse
 int launch_five_tables(const MidBoard* d_boards, int n, int kmax, void* d_masks, pp_stream s);
 // the same for the n boards d_boards[slots[i]] (slots: host array, passed in
 // the launches' parameters, kSlotBatch per launch)
+// the sliced masks of npacks packs, boards d_boards[16 p .. 16 p + 16)
+int launch_five_tables_packs(const MidBoard* d_boards, int npacks, int kmax, void* d_masks, pp_stream s);
 constexpr int kSlotBatch = 1024;
 int launch_five_tables_slots(const MidBoard* d_boards, const uint16_t* slots, int n, int kmax, void* d_masks,
                              pp_stream s);
@@ -362,8 +378,18 @@ int persistent_midgame_blocks(int ctas_per_sm, bool half = false);  // co-reside
 int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
                               pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
                               const void* d_masks, int parity = -1);
+// The same for packs; the final level's launch also writes the roots' values.
+int launch_pack_level(const MidBoard* d_boards, const MidSeg* d_segs, int nsegs, uint32_t blocks, pp_super* d_table,
+                      pp_super* d_out, int final_level, pp_stream s, const void* d_masks, uint32_t seg_blocks,
+                      int parity);
+int persistent_pack_blocks(int ctas_per_sm, bool half, bool singles);
+// every level of packs (nlevels >= 1) and of the boards left over
+int launch_pack_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
+                           const MidLevel* d_singles, int nsingles, pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
+                           const void* d_masks, int parity);
 int launch_barrier_probe(uint32_t* d_sync, uint32_t limit, pp_stream s);
 void set_barrier_spins(uint32_t polls);  // 0 = the default limit
+uint32_t barrier_spins();
 int launch_sections(const SecTask* d_tasks, int ntasks, uint32_t blocks, pp_super* d_out, pp_stream s, bool d4);
 int persistent_section_blocks(int ctas_per_sm, bool d4);
 int launch_sections_persistent(const SecTask* d_tasks, int ntasks, uint32_t blocks, pp_super* d_out,

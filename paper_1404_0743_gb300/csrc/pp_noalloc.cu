@@ -41,7 +41,7 @@ const FillLists& host_lists(int k, int mover) {
   auto it = g_host_lists.find(key);
   if (it != g_host_lists.end()) return it->second;
   FillLists L;
-  build_fill_lists(k, mover, &L);
+  build_fill_lists(k, mover, false, &L);
   return g_host_lists[key] = std::move(L);
 }
 
