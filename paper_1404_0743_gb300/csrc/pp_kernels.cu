@@ -1201,8 +1201,7 @@ template <int Q>
 __device__ __forceinline__ void line36_lines(const LineTask& tk, uint32_t gw, const uint4* qforms,
                                              pp_super* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const uint32_t group = (gw - tk.warp0) / tk.parts, part = (gw - tk.warp0) % tk.parts;
-  const uint32_t line = group * 32 + lane;
+  const uint32_t line = (gw - tk.warp0) * 32 + lane;
   const bool active = line < tk.lines;
   const uint32_t c = tk.mover;
   const uint2* __restrict__ states = reinterpret_cast<const uint2*>(c_tab.qline) + (c - 1) * kMinStates;
@@ -1233,8 +1232,8 @@ __device__ __forceinline__ void line36_lines(const LineTask& tk, uint32_t gw, co
       for (int w = 0; w < kFormWords; w++)
         if (q != Q && !line_word_used<Q>(q, w)) fc[q][w] = fo[q][w] = 0;  // never read again
   }
-  const uint32_t sq = tk.stride[Q], p1 = tk.dim[Q] * (part + 1) / tk.parts;
-  for (uint32_t p = tk.dim[Q] * part / tk.parts; p < p1; p++) {
+  const uint32_t sq = tk.stride[Q], dq = tk.dim[Q];
+  for (uint32_t p = 0; p < dq; p++) {
     const uint32_t x = __ldg(&states[tk.qoff[Q] + p]).x;  // uniform across the warp
     const uint32_t b = x & 0x1FFu, w = (x >> 9) & 0x1FFu;
     uint32_t Fc[8], Fo[8], H[8], unused[8];
@@ -1265,7 +1264,7 @@ __global__ void __launch_bounds__(kLineWarps * 32, PP_LINE_MINB)
   copy_forms(qforms, q * 512, 512);
   const uint32_t gw = blockIdx.x * kLineWarps + (threadIdx.x >> 5);
   const LineTask& tk = tasks[find_warp_owner(tasks, ntasks, gw)];
-  if (gw - tk.warp0 >= (tk.lines + 31) / 32 * tk.parts) return;  // uniform per warp (block padding)
+  if (gw - tk.warp0 >= (tk.lines + 31) / 32) return;  // uniform per warp (block padding)
   switch (q) {
     case 0: line36_lines<0>(tk, gw, qforms, out); break;
     case 1: line36_lines<1>(tk, gw, qforms, out); break;
@@ -1292,8 +1291,7 @@ template <int Q>
 __device__ __forceinline__ void ready_lines(const LineTask& tk, uint32_t gw, const uint4* qforms,
                                             pp_super* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const uint32_t group = (gw - tk.warp0) / tk.parts, part = (gw - tk.warp0) % tk.parts;
-  const uint32_t line = group * 32 + lane;
+  const uint32_t line = (gw - tk.warp0) * 32 + lane;
   const bool active = line < tk.lines;
   const uint32_t c = tk.mover;  // the parents' mover
   const uint2* __restrict__ states = reinterpret_cast<const uint2*>(c_tab.qline) + (c - 1) * kMinStates;
@@ -1321,10 +1319,10 @@ __device__ __forceinline__ void ready_lines(const LineTask& tk, uint32_t gw, con
       for (int w = 0; w < kFormWords; w++)
         if (q != Q && !line_word_used<Q>(q, w)) fc[q][w] = 0;  // never read again
   }
-  const uint32_t sq = tk.stride[Q], p1 = tk.dim[Q] * (part + 1) / tk.parts;
+  const uint32_t sq = tk.stride[Q], dq = tk.dim[Q];
   const pp_super* in = tk.child + base;
   pp_super* dst = out + tk.out + base;
-  for (uint32_t p = tk.dim[Q] * part / tk.parts; p < p1; p++) {
+  for (uint32_t p = 0; p < dq; p++) {
     const uint32_t x = __ldg(&states[tk.qoff[Q] + p]).x;  // uniform across the warp
     uint32_t H[8], unused[8], W[8], N[8], RW[8], RN[8];
     if (active) load_super32(in + (uint64_t)p * sq, W, N);
@@ -1352,7 +1350,7 @@ __global__ void __launch_bounds__(kLineWarps * 32, PP_LINE_MINB)
   copy_forms(qforms, q * 512, 512);
   const uint32_t gw = blockIdx.x * kLineWarps + (threadIdx.x >> 5);
   const LineTask& tk = tasks[find_warp_owner(tasks, ntasks, gw)];
-  if (gw - tk.warp0 >= (tk.lines + 31) / 32 * tk.parts) return;  // uniform per warp (block padding)
+  if (gw - tk.warp0 >= (tk.lines + 31) / 32) return;  // uniform per warp (block padding)
   switch (q) {
     case 0: ready_lines<0>(tk, gw, qforms, out); break;
     case 1: ready_lines<1>(tk, gw, qforms, out); break;
