@@ -954,6 +954,60 @@ struct Line35Work {
   std::vector<std::pair<int, uint64_t>> others;
 };
 
+// Longest lines first (a block's time grows with its line length, so the
+// launch ends on short ones); blocks never mix line axes (each copies its
+// axis's forms into shared memory).  With split, where the lines alone do not
+// fill the device once (20 warps on each of 152 SMs), the walked states are
+// cut into equal ranges, none below 16 states: a range evaluates the lines
+// that miss the axis again, two steps' work (one slice-35 section of 594,000
+// boards: 91 -> 41 us; cutting a pass of 11,000 warps cost it 5%).  Returns
+// the warps.
+constexpr uint32_t kLineWarpsWanted = 3040, kLineMinStates = 16;
+
+uint32_t lay_out_lines(std::vector<LineTask>* tasks, bool split) {
+  uint32_t range = 512;  // more than any list of states
+  auto warps_at = [&](uint32_t states) {
+    uint64_t n = 0;
+    for (const auto& t : *tasks) n += (uint64_t)((t.lines + 31) / 32) * ((t.dim[t.q] + states - 1) / states);
+    return n;
+  };
+  while (split && range > kLineMinStates && warps_at(range) < kLineWarpsWanted) range /= 2;
+  for (auto& t : *tasks) t.parts = (t.dim[t.q] + range - 1) / range;
+  auto steps = [](const LineTask& t) { return (t.dim[t.q] + t.parts - 1) / t.parts; };
+  std::stable_sort(tasks->begin(), tasks->end(), [&](const LineTask& a, const LineTask& b) {
+    return steps(a) != steps(b) ? steps(a) > steps(b) : a.q < b.q;
+  });
+  uint32_t warp = 0;
+  for (size_t i = 0; i < tasks->size(); i++) {
+    LineTask& t = (*tasks)[i];
+    if (i > 0 && t.q != (*tasks)[i - 1].q) warp = (warp + kLineWarps - 1) / kLineWarps * kLineWarps;
+    t.warp0 = warp;
+    warp += (t.lines + 31) / 32 * t.parts;
+  }
+  return warp;
+}
+
+// The line task of section d along its quadrant with the most states (the
+// latest of equals, so that lanes step through quadrant 0 and a warp's
+// accesses fall on neighbouring values).
+int longest_line_task(const pp_section_desc& d, LineTask* tk) {
+  const HostTables& t = host_tables();
+  uint64_t size = 1;
+  int Q = 3;
+  for (int q = 0; q < 4; q++) {
+    tk->dim[q] = d.dim[q];
+    tk->stride[q] = (uint32_t)size;
+    tk->qoff[q] = (uint16_t)t.qoff[d.bw[q][0]][d.bw[q][1]];
+    size *= d.dim[q];
+  }
+  for (int q = 2; q >= 0; q--)
+    if (d.dim[q] > d.dim[Q]) Q = q;
+  if (size >= (1ull << 32)) return fail(PP_EINVAL, "section too large");
+  tk->lines = (uint32_t)(size / d.dim[Q]);
+  tk->q = (uint32_t)Q;
+  return PP_OK;
+}
+
 int build_line35(const std::vector<pp_section_desc>& secs, const std::vector<int>& which,
                  const pp_super* in_values, const pp_super* const* child_ptrs, bool compact, Line35Work* W,
                  bool d4 = false) {
@@ -1027,66 +1081,26 @@ int build_line35(const std::vector<pp_section_desc>& secs, const std::vector<int
     start += size;
     tasks.push_back(tk);
   }
-  // A block's time grows with its line length: the longest lines start
-  // first, so the launch ends on short ones.  Blocks never mix line axes
-  // (each copies its axis's forms into shared memory).
-  std::stable_sort(tasks.begin(), tasks.end(), [](const LineTask& a, const LineTask& b) {
-    return a.dim[a.q] != b.dim[b.q] ? a.dim[a.q] > b.dim[b.q] : a.q < b.q;
-  });
-  uint32_t warp = 0;
-  for (size_t i = 0; i < tasks.size(); i++) {
-    if (i > 0 && tasks[i].q != tasks[i - 1].q) warp = (warp + kLineWarps - 1) / kLineWarps * kLineWarps;
-    tasks[i].warp0 = warp;
-    warp += (tasks[i].lines + 31) / 32;
-  }
-  W->warps = warp;
+  W->warps = lay_out_lines(&tasks, true);
   W->all = std::move(tasks);
   return PP_OK;
 }
 
-// Slice 36 by lines: no children; the line axis of a section is its
-// quadrant with the most states (the latest of equals, so that lanes step
-// through quadrant 0 and a warp's stores fall on neighbouring values).
+// Slice 36 by lines: no children.
 int build_line36(const std::vector<pp_section_desc>& secs, const std::vector<int>& which, bool compact,
                  Line35Work* W) {
-  const HostTables& t = host_tables();
-  std::vector<LineTask> tasks;
   uint64_t start = 0;
   W->terminal = true;
   for (int si : which) {
     const pp_section_desc& d = secs[si];
     LineTask tk{};
-    uint64_t size = 1, stride = 1;
-    int Q = 3;
-    for (int q = 0; q < 4; q++) {
-      tk.dim[q] = d.dim[q];
-      tk.stride[q] = (uint32_t)stride;
-      stride *= d.dim[q];
-      tk.qoff[q] = (uint16_t)t.qoff[d.bw[q][0]][d.bw[q][1]];
-      size *= d.dim[q];
-    }
-    for (int q = 2; q >= 0; q--)
-      if (d.dim[q] > d.dim[Q]) Q = q;
-    if (size >= (1ull << 32)) return fail(PP_EINVAL, "section too large");
-    tk.lines = (uint32_t)(size / d.dim[Q]);
+    if (int rc = longest_line_task(d, &tk)) return rc;
     tk.mover = 1;  // slice 36: 18 black, 18 white, black to move
     tk.out = compact ? start : d.offset;
-    tk.q = (uint32_t)Q;
-    start += size;
-    tasks.push_back(tk);
+    start += section_boards(d);
+    W->all.push_back(tk);
   }
-  // longest lines first; blocks never mix line axes
-  std::stable_sort(tasks.begin(), tasks.end(), [](const LineTask& a, const LineTask& b) {
-    return a.dim[a.q] != b.dim[b.q] ? a.dim[a.q] > b.dim[b.q] : a.q < b.q;
-  });
-  uint32_t warp = 0;
-  for (size_t i = 0; i < tasks.size(); i++) {
-    if (i > 0 && tasks[i].q != tasks[i - 1].q) warp = (warp + kLineWarps - 1) / kLineWarps * kLineWarps;
-    tasks[i].warp0 = warp;
-    warp += (tasks[i].lines + 31) / 32;
-  }
-  W->warps = warp;
-  W->all = std::move(tasks);
+  W->warps = lay_out_lines(&W->all, false);
   return PP_OK;
 }
 
@@ -1410,7 +1424,6 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
     if (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
       return fail(PP_EINVAL, "ready children: run these arguments once outside stream capture first");
   }
-  const HostTables& t = host_tables();
   uint64_t total = 0;
   const auto& secs = d4 ? slice_sections_d4(n + 1, &total) : slice_sections(n + 1, &total);
   std::vector<LineTask> tasks;
@@ -1420,27 +1433,15 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
     const uint64_t at = in_offsets ? in_offsets[i] : d.offset;
     if (at == PP_ABSENT) continue;
     LineTask tk{};
-    uint64_t size = 1, stride = 1;
-    int Q = 3;
-    for (int q = 0; q < 4; q++) {
-      tk.dim[q] = d.dim[q];
-      tk.stride[q] = (uint32_t)stride;
-      stride *= d.dim[q];
-      tk.qoff[q] = (uint16_t)t.qoff[d.bw[q][0]][d.bw[q][1]];
-      size *= d.dim[q];
-    }
-    for (int q = 2; q >= 0; q--)
-      if (d.dim[q] > d.dim[Q]) Q = q;
+    const uint64_t size = section_boards(d);
     if (at > in_count || size > in_count - at)
       return fail(PP_EINVAL, "section %zu of slice %d lies past the %llu values given", i, n + 1,
                   (unsigned long long)in_count);
-    if (size >= (1ull << 32)) return fail(PP_EINVAL, "section too large");
+    if (int rc = longest_line_task(d, &tk)) return rc;
     spans.push_back({at, at + size});
-    tk.lines = (uint32_t)(size / d.dim[Q]);
     tk.mover = (n % 2 == 0) ? 1u : 2u;  // the parents' mover
     tk.child = in + at;
     tk.out = at;
-    tk.q = (uint32_t)Q;
     tasks.push_back(tk);
   }
   if (tasks.empty()) return PP_OK;
@@ -1448,15 +1449,7 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
   std::sort(spans.begin(), spans.end());
   for (size_t i = 1; i < spans.size(); i++)
     if (spans[i].first < spans[i - 1].second) return fail(PP_EINVAL, "two sections of the input overlap");
-  std::stable_sort(tasks.begin(), tasks.end(), [](const LineTask& a, const LineTask& b) {
-    return a.dim[a.q] != b.dim[b.q] ? a.dim[a.q] > b.dim[b.q] : a.q < b.q;
-  });
-  uint32_t warp = 0;
-  for (size_t i = 0; i < tasks.size(); i++) {
-    if (i > 0 && tasks[i].q != tasks[i - 1].q) warp = (warp + kLineWarps - 1) / kLineWarps * kLineWarps;
-    tasks[i].warp0 = warp;
-    warp += (tasks[i].lines + 31) / 32;
-  }
+  const uint32_t warp = lay_out_lines(&tasks, true);
   LineTask* d = nullptr;
   if (cached) {
     cudaError_t e = cudaMalloc((void**)&d, tasks.size() * sizeof(LineTask));
@@ -1481,6 +1474,52 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
   int rc = e ? (int)e : launch_ready(d, (int)tasks.size(), warp, out, s);
   if (d) cudaFreeAsync(d, s);
   return rc ? cuda_fail(rc, "ready children") : PP_OK;
+}
+
+// One section of slice n < 35 by lines.  Children of at most twice its boards
+// are first turned into ready records in a stream-ordered temporary (19 ps a
+// value), which table_line_kernel reads (27 ps a board) where the raw kernel
+// takes about 80 ps a board, and more on a small section: it has one warp for
+// 32 whole lines.
+int run_one_section(int n, SecTask tk, pp_super* out, pp_stream s) {
+  const HostTables& t = host_tables();
+  std::vector<LineTask> kids;
+  uint64_t total = 0, at[4] = {};
+  for (int q = 0; q < 4; q++) {
+    if (!(tk.movable >> q & 1)) continue;
+    pp_section_desc d{};
+    std::memcpy(d.bw, tk.bw, sizeof d.bw);
+    d.bw[q][tk.mover - 1]++;
+    for (int r = 0; r < 4; r++) d.dim[r] = (uint16_t)t.qdim[d.bw[r][0]][d.bw[r][1]];
+    LineTask l{};
+    if (section_boards(d) > 2 * tk.size || longest_line_task(d, &l)) return run_section_lines({tk}, false, out, s);
+    l.mover = tk.mover;  // the parents' mover
+    l.child = tk.child[q];
+    l.out = at[q] = total;
+    total += section_boards(d);
+    kids.push_back(l);
+  }
+  pp_super* prep = nullptr;
+  if (!total || total > 2 * tk.size || cudaMallocAsync((void**)&prep, total * sizeof(pp_super), s) != cudaSuccess) {
+    cudaGetLastError();  // no room for the temporary: read the children as they are
+    return run_section_lines({tk}, false, out, s);
+  }
+  const uint32_t warps = lay_out_lines(&kids, true);
+  LineTask* d = nullptr;
+  cudaError_t e = cudaMallocAsync((void**)&d, kids.size() * sizeof(LineTask), s);
+  if (!e) e = cudaMemcpyAsync(d, kids.data(), kids.size() * sizeof(LineTask), cudaMemcpyHostToDevice, s);
+  int rc = e ? (int)e : launch_ready(d, (int)kids.size(), warps, prep, s);
+  if (d) cudaFreeAsync(d, s);
+  if (rc) {
+    cudaFreeAsync(prep, s);
+    return cuda_fail(rc, "ready children");
+  }
+  for (int q = 0; q < 4; q++)
+    if (tk.movable >> q & 1) tk.child[q] = prep + at[q];
+  tk.prepared = 2;
+  rc = run_section_lines({tk}, false, out, s);
+  cudaFreeAsync(prep, s);
+  return rc;
 }
 
 int slice_step(int n, const pp_super* in_values, pp_super* out_values, const uint8_t* filter,
@@ -1558,8 +1597,7 @@ int pp_section_compute(int n, const pp_section_desc* parent, const pp_super* con
   uint32_t blocks = 0;
   int rc = build_tasks(n, one, {0}, nullptr, d_child ? d_child : none, true, &tasks, &blocks);
   if (rc) return rc;
-  if (n < 35) return run_section_lines(tasks, false, d_out, s);
-  return run_tasks(tasks, blocks, d_out, s);
+  return run_one_section(n, tasks[0], d_out, s);
 }
 
 int pp_section_compute_desc(int n, const pp_section_desc* parent, const pp_super* const d_child[4],

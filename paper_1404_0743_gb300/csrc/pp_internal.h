@@ -316,7 +316,7 @@ struct LineTask {
   uint32_t mover;         // 1 black, 2 white
   uint32_t cqoff;         // qlist offset of quadrant q's counts in the child section
   uint32_t q;             // the line axis (the non-full quadrant); every block holds one q
-  uint32_t pad;
+  uint32_t parts;         // equal ranges of Q's states, a warp each (slice 35 and the ready pass; else 1)
 };
 #ifndef PP_LINE_WARPS
 #define PP_LINE_WARPS 4

@@ -1030,7 +1030,8 @@ template <int Q, bool ONDEMAND>
 __device__ __forceinline__ void line35_lines(const LineTask& tk, uint32_t gw, const uint4* qforms, uint32_t* cold,
                                              pp_super* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const uint32_t line = (gw - tk.warp0) * 32 + lane;
+  const uint32_t group = (gw - tk.warp0) / tk.parts, part = (gw - tk.warp0) % tk.parts;
+  const uint32_t line = group * 32 + lane;
   const bool active = line < tk.lines;
   const uint32_t c = tk.mover;
   const uint2* __restrict__ moves = reinterpret_cast<const uint2*>(c_tab.qline) + (c - 1) * kMinStates;
@@ -1082,10 +1083,11 @@ __device__ __forceinline__ void line35_lines(const LineTask& tk, uint32_t gw, co
   const uint4* __restrict__ sorted = reinterpret_cast<const uint4*>(c_tab.qsorted) + (c - 1) * kMinStates + tk.qoff[Q];
   // the current child's tables A, Y2, Y3, already turned ucur along Q
   uint32_t A[8], Y2[8], Y3[8], jprev = 0xFFFFFFFFu, ucur = 0;
-  uint4 mnext = __ldg(sorted);
-  for (uint32_t k = 0; k < dq; k++) {
+  const uint32_t k1 = dq * (part + 1) / tk.parts;
+  uint4 mnext = __ldg(sorted + dq * part / tk.parts);
+  for (uint32_t k = dq * part / tk.parts; k < k1; k++) {
     const uint4 m = mnext;  // uniform across the warp
-    if (k + 1 < dq) mnext = __ldg(sorted + k + 1);
+    if (k + 1 < k1) mnext = __ldg(sorted + k + 1);
     const uint32_t j = (m.y >> 4) & 0x1FFu;
     if (j != jprev) {
       // the child: this lane's fixed quadrants and the child count class's
@@ -1177,7 +1179,7 @@ __global__ void __launch_bounds__(kLineWarps * 32, PP_LINE_MINB)
   copy_forms(qforms, q * 512, 512);
   const uint32_t gw = blockIdx.x * kLineWarps + (threadIdx.x >> 5);
   const LineTask& tk = tasks[find_warp_owner(tasks, ntasks, gw)];
-  if (gw - tk.warp0 >= (tk.lines + 31) / 32) return;  // uniform per warp (block padding)
+  if (gw - tk.warp0 >= (tk.lines + 31) / 32 * tk.parts) return;  // uniform per warp (block padding)
   switch (q) {
     case 0: line35_lines<0, ONDEMAND>(tk, gw, qforms, cold, out); break;
     case 1: line35_lines<1, ONDEMAND>(tk, gw, qforms, cold, out); break;
@@ -1291,7 +1293,8 @@ template <int Q>
 __device__ __forceinline__ void ready_lines(const LineTask& tk, uint32_t gw, const uint4* qforms,
                                             pp_super* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const uint32_t line = (gw - tk.warp0) * 32 + lane;
+  const uint32_t group = (gw - tk.warp0) / tk.parts, part = (gw - tk.warp0) % tk.parts;
+  const uint32_t line = group * 32 + lane;
   const bool active = line < tk.lines;
   const uint32_t c = tk.mover;  // the parents' mover
   const uint2* __restrict__ states = reinterpret_cast<const uint2*>(c_tab.qline) + (c - 1) * kMinStates;
@@ -1319,10 +1322,10 @@ __device__ __forceinline__ void ready_lines(const LineTask& tk, uint32_t gw, con
       for (int w = 0; w < kFormWords; w++)
         if (q != Q && !line_word_used<Q>(q, w)) fc[q][w] = 0;  // never read again
   }
-  const uint32_t sq = tk.stride[Q], dq = tk.dim[Q];
+  const uint32_t sq = tk.stride[Q], p1 = tk.dim[Q] * (part + 1) / tk.parts;
   const pp_super* in = tk.child + base;
   pp_super* dst = out + tk.out + base;
-  for (uint32_t p = 0; p < dq; p++) {
+  for (uint32_t p = tk.dim[Q] * part / tk.parts; p < p1; p++) {
     const uint32_t x = __ldg(&states[tk.qoff[Q] + p]).x;  // uniform across the warp
     uint32_t H[8], unused[8], W[8], N[8], RW[8], RN[8];
     if (active) load_super32(in + (uint64_t)p * sq, W, N);
@@ -1350,7 +1353,7 @@ __global__ void __launch_bounds__(kLineWarps * 32, PP_LINE_MINB)
   copy_forms(qforms, q * 512, 512);
   const uint32_t gw = blockIdx.x * kLineWarps + (threadIdx.x >> 5);
   const LineTask& tk = tasks[find_warp_owner(tasks, ntasks, gw)];
-  if (gw - tk.warp0 >= (tk.lines + 31) / 32) return;  // uniform per warp (block padding)
+  if (gw - tk.warp0 >= (tk.lines + 31) / 32 * tk.parts) return;  // uniform per warp (block padding)
   switch (q) {
     case 0: ready_lines<0>(tk, gw, qforms, out); break;
     case 1: ready_lines<1>(tk, gw, qforms, out); break;
