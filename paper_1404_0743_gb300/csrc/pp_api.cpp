@@ -144,6 +144,12 @@ int describe_board(uint64_t packed, int max_empty, MidBoard* mb, int i) {
 #define PP_PACK_MIN_EMPTY 7
 #endif
 constexpr int kPackMinEmpty = PP_PACK_MIN_EMPTY;
+// Where boards are left over, a batch pays for both kinds of masks and runs
+// the single boards at the packs' occupancy, 10-20 us that fewer packed fills
+// than this don't win back (40 boards: with 10 empty cells, 0.57 million
+// fills in packs, 115 us against 106 all one by one; with 11, 1.6 million,
+// 160 against 169; 72 with 10, 1.1 million, the same).
+constexpr uint64_t kPackMinFills = 1250000;
 
 std::map<std::tuple<int, int, bool>, std::unique_ptr<LevelLists>> g_lists;
 
@@ -270,13 +276,17 @@ struct pp_midgame_plan {
   int n = 0, max_empty = 0, kmax = 0;
   uint64_t table_entries = 0;  // compact fill-table entries of all boards
   void* d_mem = nullptr;  // one allocation holding the four arrays below
-  MidBoard* d_boards = nullptr;  // the packs' boards, then the others
+  MidBoard* d_boards = nullptr;  // the packs' boards, the ones solved one by one, the small ones
   MidSeg* d_segs = nullptr;
   using Level = MidLevel;
   // packs of boards of one shape, and the boards left over one by one: each
-  // with its own levels, levels[j] being stones added m = kmax - j
-  int npacks = 0, pack_kmax = 0;
+  // with its own levels, levels[j] being stones added m = kmax - j; then the
+  // boards solved in one block each
+  int npacks = 0, pack_kmax = 0, nsmall = 0;
+  const SmallShape* d_shapes = nullptr;
+  size_t small_smem = 0;
   std::vector<Level> pack_levels, levels;
+  bool uses_barrier() const { return mode == 1 && (npacks || !levels.empty()); }
   MidLevel* d_pack_levels = nullptr;
   MidLevel* d_levels = nullptr;
   uint32_t* d_sync = nullptr;  // barrier count, generation, status (persistent mode)
@@ -421,31 +431,56 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
   // mover), then the other boards in their given order
   {
     int taken[kMaxEmpty + 1] = {}, in_packs[kMaxEmpty + 1], first[kMaxEmpty + 1];
-    int at = 0;
-    for (int k = kMaxEmpty; k >= 0; k--) {
+    int at = 0, alone = 0;
+    uint64_t packed_fills = 0;
+    for (int k = 0; k <= kMaxEmpty; k++) {
       in_packs[k] = k >= kPackMinEmpty ? per_k[k] / kPackBoards * kPackBoards : 0;
+      packed_fills += (uint64_t)in_packs[k] * fills_total(k);
+      if (k > kSmallEmpty) alone += per_k[k] - in_packs[k];
+    }
+    if (alone && packed_fills < kPackMinFills) std::fill(in_packs, in_packs + kMaxEmpty + 1, 0);
+    for (int k = kMaxEmpty; k >= 0; k--) {
       first[k] = at;
       at += in_packs[k];
       if (in_packs[k]) P->pack_kmax = std::max(P->pack_kmax, k);
     }
     P->npacks = at / kPackBoards;
     std::vector<MidBoard> sorted(n);
+    int small = n;  // the small ones fill the end
     for (const MidBoard& b : boards) {
       const int k = (int)b.k;
-      sorted[taken[k] < in_packs[k] ? first[k] + taken[k] : at++] = b;
+      sorted[taken[k] < in_packs[k] ? first[k] + taken[k] : k <= kSmallEmpty ? --small : at++] = b;
       taken[k]++;
     }
+    P->nsmall = n - small;
     boards = std::move(sorted);
   }
+  const int nsingle = n - P->nsmall;  // where the small ones start
   for (int i = 0; i < n; i++) {
     boards[i].table = P->table_entries;  // boards' compact tables back to back
     P->table_entries += fills_total((int)boards[i].k);
     boards[i].masks = (uint64_t)i * mask_entries_per_board(max_empty);
-    if (i >= P->npacks * kPackBoards) P->kmax = std::max(P->kmax, (int)boards[i].k);
+    if (i >= P->npacks * kPackBoards && i < nsingle) P->kmax = std::max(P->kmax, (int)boards[i].k);
   }
   std::vector<MidSeg> segs;
+  std::vector<SmallShape> shapes(P->nsmall ? kSmallEmpty + 1 : 0);
   {
     std::lock_guard<std::mutex> lock(g_mutex);
+    for (int i = nsingle; i < n; i++) {
+      SmallShape& S = shapes[boards[i].k];  // its number of empty cells decides the mover
+      if (S.list) continue;
+      const int k = (int)boards[i].k;
+      std::string err;
+      const LevelLists* L = level_lists(k, (int)boards[i].mover, &err);
+      if (!L) return fail(PP_ECUDA, "%s", err.c_str());
+      S.list = L->d_entries;
+      S.ranks = L->d_ranks;
+      for (int m = 0; m <= k; m++) S.off[m] = (uint32_t)L->offset[m], S.ranks_at[m] = (uint32_t)L->ranks_at[m];
+      S.off[k + 1] = (uint32_t)L->total;
+      S.nranks = S.ranks_at[k];  // a full board has no moves
+      P->small_smem = std::max(P->small_smem, midgame_small_bytes(k, S.off[k + 1], S.nranks));
+    }
+    if (P->small_smem > kSmallSmem) return fail(PP_ECUDA, "small boards need %zu bytes of shared memory", P->small_smem);
     // One level's descriptors: units are packs (their first boards) or single
     // boards, `per_block` fills to a block.  When all are of one shape a
     // level has one shared descriptor, unit j being the j-th.
@@ -496,7 +531,7 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     };
     const int packed = P->npacks * kPackBoards;
     int rc = add_levels(0, P->npacks, kPackBoards, kPackFills, true, P->pack_kmax, &P->pack_levels);
-    if (!rc) rc = add_levels(packed, n - packed, 1, kBlock, false, P->kmax, &P->levels);
+    if (!rc) rc = add_levels(packed, nsingle - packed, 1, kBlock, false, P->kmax, &P->levels);
     if (rc) return rc;
   }
   if (n > 0) {
@@ -506,10 +541,12 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     const size_t ob = 0, os = ob + up(boards.size() * sizeof(MidBoard));
     const size_t op = os + up(segs.size() * sizeof(MidSeg));
     const size_t ol = op + up(P->pack_levels.size() * sizeof(MidLevel));
-    const size_t oy = ol + up(P->levels.size() * sizeof(MidLevel)), total = oy + 4 * sizeof(uint32_t);
+    const size_t oh = ol + up(P->levels.size() * sizeof(MidLevel));
+    const size_t oy = oh + up(shapes.size() * sizeof(SmallShape)), total = oy + 4 * sizeof(uint32_t);
     std::vector<char> pack(total, 0);
     std::memcpy(pack.data() + ob, boards.data(), boards.size() * sizeof(MidBoard));
-    std::memcpy(pack.data() + os, segs.data(), segs.size() * sizeof(MidSeg));
+    if (!segs.empty()) std::memcpy(pack.data() + os, segs.data(), segs.size() * sizeof(MidSeg));
+    if (!shapes.empty()) std::memcpy(pack.data() + oh, shapes.data(), shapes.size() * sizeof(SmallShape));
     if (!P->pack_levels.empty())
       std::memcpy(pack.data() + op, P->pack_levels.data(), P->pack_levels.size() * sizeof(MidLevel));
     if (!P->levels.empty()) std::memcpy(pack.data() + ol, P->levels.data(), P->levels.size() * sizeof(MidLevel));
@@ -536,6 +573,7 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     P->d_segs = reinterpret_cast<MidSeg*>(base + os);
     P->d_pack_levels = reinterpret_cast<MidLevel*>(base + op);
     P->d_levels = reinterpret_cast<MidLevel*>(base + ol);
+    P->d_shapes = reinterpret_cast<SmallShape*>(base + oh);
     P->d_sync = reinterpret_cast<uint32_t*>(base + oy);
   }
   *plan = P.release();
@@ -547,16 +585,19 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
 
 namespace {
 
-int launch_masks(const pp_midgame_plan* P, void* masks, pp_stream s) {
-  const int packed = P->npacks * kPackBoards;
-  int rc = launch_five_tables_packs(P->d_boards, P->npacks, P->pack_kmax, masks, s);
-  if (!rc) rc = launch_five_tables(P->d_boards + packed, P->n - packed, P->kmax, masks, s);
+// The small boards, whole, and the other boards' masks.
+int launch_small_and_masks(const pp_midgame_plan* P, void* masks, pp_super* d_out, pp_stream s) {
+  const int packed = P->npacks * kPackBoards, singles = P->n - P->nsmall - packed;
+  int rc = launch_midgame_small(P->d_boards + packed + singles, P->nsmall, P->d_shapes, P->small_smem, d_out,
+                                P->parity, s);
+  if (!rc) rc = launch_five_tables_packs(P->d_boards, P->npacks, P->pack_kmax, masks, s);
+  if (!rc) rc = launch_five_tables(P->d_boards + packed, singles, P->kmax, masks, s);
   return rc;
 }
 
 // One launch per level: the packs' levels, then the other boards'.
 int launch_levels(const pp_midgame_plan* P, void* d_workspace, void* masks, pp_super* d_out, pp_stream s) {
-  int rc = launch_masks(P, masks, s);
+  int rc = launch_small_and_masks(P, masks, d_out, s);
   for (const bool packs : {true, false}) {
     const auto& levels = packs ? P->pack_levels : P->levels;
     for (size_t j = 0; !rc && j < levels.size(); j++) {
@@ -571,10 +612,11 @@ int launch_levels(const pp_midgame_plan* P, void* d_workspace, void* masks, pp_s
   return rc;
 }
 
-// Kernels of launch_levels: masks and levels of either kind, and the packs'
-// root values.
+// Kernels of launch_levels: masks and levels of either kind, the packs' root
+// values, and the small boards.
 uint64_t level_launches(const pp_midgame_plan* P) {
-  return (P->npacks ? P->pack_levels.size() + 2 : 0) + (P->levels.empty() ? 0 : P->levels.size() + 1);
+  return (P->npacks ? P->pack_levels.size() + 2 : 0) + (P->levels.empty() ? 0 : P->levels.size() + 1) +
+         (P->nsmall ? 1 : 0);
 }
 
 }  // namespace
@@ -592,15 +634,14 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
   // workspace: fill tables of all boards, then their five tables
   void* masks = (char*)d_workspace + (size_t)P->table_entries * fill_entry_bytes(P->parity);
   if (P->mode == 1) {
-    cudaError_t e = cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s);
-    if (e) return cuda_fail(e, "barrier reset");
-    int rc = launch_masks(P, masks, s);
+    int rc = launch_small_and_masks(P, masks, d_out, s);
+    if (!rc && P->uses_barrier()) rc = (int)cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s);
     const bool half = P->parity >= 0;
     if (!rc && P->npacks)
       rc = launch_pack_persistent(P->d_boards, P->d_segs, P->d_pack_levels, (int)P->pack_levels.size(), P->d_levels,
                                   (int)P->levels.size(), (pp_super*)d_workspace, d_out, P->d_sync,
                                   persistent_pack_blocks(P->ctas_per_sm, half, !P->levels.empty()), s, masks, P->parity);
-    else if (!rc)
+    else if (!rc && !P->levels.empty())
       rc = launch_midgame_persistent(P->d_boards, P->d_segs, P->d_levels, (int)P->levels.size(),
                                      (pp_super*)d_workspace, d_out, P->d_sync,
                                      persistent_midgame_blocks(P->ctas_per_sm, half), s, masks, P->parity);
@@ -784,7 +825,8 @@ int solve_device(const uint64_t* d_boards, int n, pp_super* d_out, int max_empty
   if (!rc) one_shot_mode(P);
   if (!rc) rc = pp_midgame_plan_run(P, d_workspace, ws_bytes, d_out, s);
   uint32_t st = 0;
-  cudaError_t e = rc ? cudaSuccess : cudaMemcpyAsync(&st, P->d_sync + 2, sizeof st, cudaMemcpyDeviceToHost, s);
+  cudaError_t e = cudaSuccess;
+  if (!rc && P->uses_barrier()) e = cudaMemcpyAsync(&st, P->d_sync + 2, sizeof st, cudaMemcpyDeviceToHost, s);
   pp_midgame_plan_destroy(P);
   if (!e) e = cudaStreamSynchronize(s);
   if (!rc && e) rc = cuda_fail(e, "midgame solve");
@@ -825,7 +867,7 @@ int pp_midgame_solve_host(const uint64_t* h_boards, int n, pp_super* h_out, int 
   uint32_t st = 0;
   cudaError_t e = cudaSuccess;
   if (!rc) e = cudaMemcpyAsync(h_out, d_out, n * sizeof(pp_super), cudaMemcpyDeviceToHost, s);
-  if (!rc && !e) e = cudaMemcpyAsync(&st, P->d_sync + 2, sizeof st, cudaMemcpyDeviceToHost, s);
+  if (!rc && !e && P->uses_barrier()) e = cudaMemcpyAsync(&st, P->d_sync + 2, sizeof st, cudaMemcpyDeviceToHost, s);
   pp_midgame_plan_destroy(P);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (!rc && (e || e2)) rc = cuda_fail(e ? e : e2, "midgame solve (host arrays)");

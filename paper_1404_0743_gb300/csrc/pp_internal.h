@@ -214,6 +214,18 @@ struct MidLevel {
 // derives the rest from the block index.
 constexpr uint32_t kSharedSegs = 0x80000000u;
 
+// Lists of the boards solved in one block each (midgame_small_kernel), by
+// number of empty cells: off[m] = fills below level m, off[k + 1] all of them.
+constexpr int kSmallEmpty = 7;
+constexpr size_t kSmallSmem = 96 << 10;  // what the largest of them may need
+struct SmallShape {
+  const uint64_t* list;
+  const uint32_t* ranks;
+  uint32_t off[kSmallEmpty + 2];
+  uint32_t ranks_at[kSmallEmpty + 1];
+  uint32_t nranks;
+};
+
 // Boards of one shape solved together, their tables sliced across them
 // (pack_level_kernel).  A pack's boards have consecutive descriptors; its
 // records and masks take the room of the boards' own, from the first's.  A
@@ -378,6 +390,10 @@ int persistent_midgame_blocks(int ctas_per_sm, bool half = false);  // co-reside
 int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
                               pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
                               const void* d_masks, int parity = -1);
+// n boards with at most kSmallEmpty empty cells; smem: the most midgame_small_bytes of them
+int launch_midgame_small(const MidBoard* d_boards, int n, const SmallShape* d_shapes, size_t smem, pp_super* d_out,
+                         int parity, pp_stream s);
+size_t midgame_small_bytes(int k, uint32_t fills, uint32_t nranks);
 // The same for packs; the final level's launch also writes the roots' values.
 int launch_pack_level(const MidBoard* d_boards, const MidSeg* d_segs, int nsegs, uint32_t blocks, pp_super* d_table,
                       pp_super* d_out, int final_level, pp_stream s, const void* d_masks, uint32_t seg_blocks,

@@ -612,6 +612,110 @@ __global__ void five_table_pack_kernel(const MidBoard* __restrict__ boards, int 
   }
 }
 
+// ---------------------------------------------------------------------------
+// Boards with few empty cells, one block to a board: lists, masks and every
+// record in shared memory, levels divided by block barriers (paper, "Open
+// source and data").  The launch-wide kernels spend such a solve on grid
+// barriers and round trips to L2.  Records are 80 bytes apart, so that 16-byte
+// reads of unrelated records spread over the banks.
+// ---------------------------------------------------------------------------
+constexpr int kSmallPitch = 5;  // 16-byte units per record
+
+__host__ __device__ inline size_t small_bytes(int k, uint32_t fills, uint32_t nranks) {
+  return (size_t)fills * (kSmallPitch * 16 + sizeof(uint64_t)) + ((size_t)2 << k) * 32 + (size_t)nranks * sizeof(uint32_t);
+}
+
+__global__ void __launch_bounds__(kBlock) midgame_small_kernel(const MidBoard* __restrict__ boards,
+                                                               const SmallShape* __restrict__ shapes,
+                                                               pp_super* __restrict__ out, int parity) {
+  extern __shared__ uint4 small_smem[];
+  __shared__ SmallShape S;
+  __shared__ MidBoard B;
+  const uint32_t tid = threadIdx.x;
+  if (tid < sizeof(MidBoard) / 4)
+    reinterpret_cast<uint32_t*>(&B)[tid] = reinterpret_cast<const uint32_t*>(boards + blockIdx.x)[tid];
+  const int k = (int)boards[blockIdx.x].k;
+  if (tid < sizeof(SmallShape) / 4)
+    reinterpret_cast<uint32_t*>(&S)[tid] = reinterpret_cast<const uint32_t*>(shapes + k)[tid];
+  __syncthreads();
+  const uint32_t fills = S.off[k + 1], kk = 1u << k;
+  uint4* masks = small_smem;                                   // [colour][subset], two units each
+  uint4* rec = masks + 4 * kk;                                 // [fill], kSmallPitch units each
+  uint64_t* list = reinterpret_cast<uint64_t*>(rec + (size_t)kSmallPitch * fills);
+  uint32_t* ranks = reinterpret_cast<uint32_t*>(list + fills);
+  for (uint32_t i = tid; i < fills; i += kBlock) list[i] = __ldg(S.list + i);
+  for (uint32_t i = tid; i < S.nranks; i += kBlock) ranks[i] = __ldg(S.ranks + i);
+  const uint32_t capb = B.mover == 1 ? (k + 1) / 2 : k / 2, capw = k - capb;
+  for (uint32_t t = tid; t < 2 * kk; t += kBlock) {
+    const uint32_t white = t >> k, subset = t & (kk - 1);
+    if (__popc(subset) > (int)(white ? capw : capb)) continue;
+    uint32_t f[4][kFormWords], F[8];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      uint32_t p = white ? B.root_w[q] : B.root_b[q];
+      for (int i = B.qstart[q]; i < B.qstart[q + 1]; i++) p |= (subset >> i & 1u) << B.slot_bit[i];
+      load_forms(q, p, f[q]);
+    }
+    five_mask(f, F);
+    masks[2 * t] = make_uint4(F[0], F[1], F[2], F[3]);
+    masks[2 * t + 1] = make_uint4(F[4], F[5], F[6], F[7]);
+  }
+  __syncthreads();
+  auto get = [](const uint4* p, uint32_t r[8]) {
+    const uint4 a = p[0], b = p[1];
+    r[0] = a.x, r[1] = a.y, r[2] = a.z, r[3] = a.w, r[4] = b.x, r[5] = b.y, r[6] = b.z, r[7] = b.w;
+  };
+  for (int level = k; level >= 0; level--) {
+    const uint32_t c = (level & 1) ? 3u - B.mover : B.mover, moves = (uint32_t)(k - level);
+    const uint32_t at = S.off[level], count = S.off[level + 1] - at;
+    for (uint32_t e = tid; e < count; e += kBlock) {
+      const uint64_t entry = list[at + e];
+      const uint32_t bm = (uint32_t)(entry >> 32) & 0xFFFFu, wm = (uint32_t)(entry >> 48);
+      uint32_t Fc[8], Fo[8], W[8], N[8];
+      const uint32_t full = moves ? 0u : 0xFFFFFFFFu;  // a full board: win F_c & ~F_o, not-lose F_c | ~F_o
+#pragma unroll
+      for (int w = 0; w < 8; w++) W[w] = 0, N[w] = full;
+      const uint32_t* rk = ranks + S.ranks_at[level] + e * moves;
+      for (uint32_t m = 0; m < moves; m++) {
+        const uint4* child = rec + (size_t)kSmallPitch * (S.off[level + 1] + rk[m]);
+        uint32_t a[8], b[8];
+        get(child, a);
+        get(child + 2, b);
+#pragma unroll
+        for (int w = 0; w < 8; w++) W[w] |= a[w], N[w] |= b[w];
+      }
+      get(masks + 2 * ((c - 1) * kk + (c == 1 ? bm : wm)), Fc);
+      get(masks + 2 * ((2 - c) * kk + (c == 1 ? wm : bm)), Fo);
+#pragma unroll
+      for (int w = 0; w < 8; w++) {
+        W[w] = ~Fo[w] & (Fc[w] | W[w]);
+        N[w] = Fc[w] | (~Fo[w] & N[w]);
+      }
+      if (level == 0) {
+        if (parity >= 0) {
+#pragma unroll
+          for (int w = 0; w < 8; w++) W[w] &= class_bits((uint32_t)parity, w), N[w] &= class_bits((uint32_t)parity, w);
+        }
+        store_super(out + B.out, W, N);
+      } else {  // the tables the parents OR (see midgame_fill)
+        uint32_t P[8], R[8];
+#pragma unroll
+        for (int w = 0; w < 8; w++) W[w] = ~W[w], N[w] = ~N[w];
+        rmax(N, P);
+        rmax(W, R);
+#pragma unroll
+        for (int w = 0; w < 8; w++) P[w] |= Fo[w], R[w] |= Fo[w];
+        uint4* r = rec + (size_t)kSmallPitch * (at + e);
+        r[0] = make_uint4(P[0], P[1], P[2], P[3]);
+        r[1] = make_uint4(P[4], P[5], P[6], P[7]);
+        r[2] = make_uint4(R[0], R[1], R[2], R[3]);
+        r[3] = make_uint4(R[4], R[5], R[6], R[7]);
+      }
+    }
+    __syncthreads();
+  }
+}
+
 template <bool HALF>
 __global__ void __launch_bounds__(kBlock, PP_MID_MINB) midgame_level_kernel(const MidBoard* __restrict__ boards,
                                                                const MidSeg* __restrict__ segs, int nsegs,
@@ -2183,6 +2287,20 @@ int launch_five_tables(const MidBoard* d_boards, int n, int kmax, void* d_masks,
   count_launch();
   return (int)cudaGetLastError();
 }
+
+int launch_midgame_small(const MidBoard* d_boards, int n, const SmallShape* d_shapes, size_t smem, pp_super* d_out,
+                         int parity, pp_stream s) {
+  if (n <= 0) return 0;
+  // more than the 48 KB of static shared memory: opt in once
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(midgame_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
+  if (attr) return (int)attr;
+  midgame_small_kernel<<<n, kBlock, smem, s>>>(d_boards, d_shapes, d_out, parity);
+  count_launch();
+  return (int)cudaGetLastError();
+}
+
+size_t midgame_small_bytes(int k, uint32_t fills, uint32_t nranks) { return small_bytes(k, fills, nranks); }
 
 int launch_five_tables_packs(const MidBoard* d_boards, int npacks, int kmax, void* d_masks, pp_stream s) {
   if (npacks <= 0) return 0;
