@@ -130,19 +130,6 @@ __device__ __forceinline__ void store_super(pp_super* p, const uint32_t W[8], co
   v[3] = make_uint4(N[4], N[5], N[6], N[7]);
 }
 
-// Child values of a level are read through L2 (__ldcg) when the reading and
-// writing levels run in the same launch: L1 is not coherent across SMs.
-template <bool L2ONLY>
-__device__ __forceinline__ void load_child(const pp_super* p, uint32_t W[8], uint32_t N[8]) {
-  if (L2ONLY) {
-    ld256_cg(p->win, W);
-    ld256_cg(p->notlose, N);
-  } else {
-    ld256_nc(p->win, W);
-    ld256_nc(p->notlose, N);
-  }
-}
-
 __device__ __forceinline__ void load_mask(const uint4* p, uint32_t F[8]) { ld256_nc(p, F); }
 
 // ---------------------------------------------------------------------------
@@ -199,8 +186,91 @@ __device__ __forceinline__ void half_unpack(const uint32_t h[4], uint32_t p, uin
 // per move and takes no rmax; each fill still takes two.  The root stores
 // its value.  A fill's own masks come from the board's colour-subset five
 // tables (five_table_kernel); its children from the level below.
-template <bool L2ONLY, bool HALF>
-__device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+//
+// Whole tables: a pair of lanes shares a fill, the even one folding the
+// children's win slots and making the fill's not-lose slot, the odd one the
+// other way round, four loads in flight each.  A warp's load of children then
+// takes 64 bytes of each line it touches (a lane to a record took 32 at a
+// time, two L1 wavefronts a record).  Still bound by the latency and the L1
+// wavefronts of scattered records: one board with 16 empty cells 635 -> 620
+// us, 400 served queries 5.77 -> 5.49 ms.
+template <bool L2ONLY>
+__device__ __forceinline__ void midgame_fill_whole(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+                                                  int nsegs, uint32_t vb, pp_super* __restrict__ table,
+                                                  pp_super* __restrict__ out, int final_level,
+                                                  const uint4* __restrict__ masks, uint32_t seg_blocks) {
+  const uint32_t per = seg_blocks & ~kSharedSegs;
+  const int owner = per ? (int)(vb / per) : find_block_owner(segs, nsegs, vb);
+  MidSeg sg = segs[(seg_blocks & kSharedSegs) ? 0 : owner];
+  if (seg_blocks & kSharedSegs) sg.board += (uint32_t)owner, sg.block0 = (uint32_t)owner * per;
+  const MidBoard& B = boards[sg.board];
+  const int k = (int)B.k, level = (int)sg.level;
+  const uint32_t c = (level & 1) ? 3u - B.mover : B.mover;  // colour to move
+  const uint4* mt = masks + 2 * B.masks;
+  const uint32_t kk = 1u << k, moves = (uint32_t)(k - level), slot = threadIdx.x & 1;
+  const char* kids = reinterpret_cast<const char*>(table + B.table + sg.coff) + 32 * slot;
+  pp_super* own = table + B.table + sg.loff;
+  auto load = [&](uint32_t child, uint32_t r[8]) {
+    if (L2ONLY)
+      ld256_cg(kids + (uint64_t)child * sizeof(pp_super), r);
+    else
+      ld256_nc(kids + (uint64_t)child * sizeof(pp_super), r);
+  };
+#pragma unroll 1
+  for (uint32_t half = 0; half < 2; half++) {
+    const uint32_t e = (vb - sg.block0) * kBlock + half * (kBlock / 2) + (threadIdx.x >> 1);
+    if (e >= sg.count) return;
+    const uint64_t entry = __ldg(sg.list + e);
+    const uint32_t* __restrict__ rk = sg.ranks + (uint64_t)e * moves;
+    uint32_t A[8];
+    const uint32_t full = slot && !moves ? 0xFFFFFFFFu : 0u;
+#pragma unroll
+    for (int w = 0; w < 8; w++) A[w] = full;
+    uint32_t m = 0;
+    for (; m + 3 < moves; m += 4) {
+      const uint32_t r0 = __ldg(rk + m), r1 = __ldg(rk + m + 1), r2 = __ldg(rk + m + 2), r3 = __ldg(rk + m + 3);
+      uint32_t a[8], b[8], x[8], y[8];
+      load(r0, a);
+      load(r1, b);
+      load(r2, x);
+      load(r3, y);
+#pragma unroll
+      for (int w = 0; w < 8; w++) A[w] |= a[w] | b[w], A[w] |= x[w] | y[w];
+    }
+    for (; m < moves; m++) {
+      uint32_t a[8];
+      load(__ldg(rk + m), a);
+#pragma unroll
+      for (int w = 0; w < 8; w++) A[w] |= a[w];
+    }
+    const uint32_t bm = (uint32_t)(entry >> 32) & 0xFFFFu, wm = (uint32_t)(entry >> 48);
+    uint32_t Fc[8], Fo[8], R[8];
+    load_mask(mt + 2 * ((c - 1) * kk + (c == 1 ? bm : wm)), Fc);
+    load_mask(mt + 2 * ((2 - c) * kk + (c == 1 ? wm : bm)), Fo);
+    const uint32_t nl = slot ? 0xFFFFFFFFu : 0u;
+#pragma unroll
+    for (int w = 0; w < 8; w++) {
+      const uint32_t mine = Fc[w] & (nl | ~Fo[w]);
+      A[w] = mine | (~Fo[w] & A[w]);
+    }
+    if (final_level || sg.final) {
+      uint4* v = reinterpret_cast<uint4*>(slot ? out[B.out].notlose : out[B.out].win);
+      v[0] = make_uint4(A[0], A[1], A[2], A[3]);
+      v[1] = make_uint4(A[4], A[5], A[6], A[7]);
+      continue;
+    }
+#pragma unroll
+    for (int w = 0; w < 8; w++) A[w] = ~A[w];
+    rmax(A, R);
+#pragma unroll
+    for (int w = 0; w < 8; w++) R[w] |= Fo[w];
+    st256(slot ? own[e].win : own[e].notlose, R);
+  }
+}
+
+// Half tables (32-byte records): one lane to a fill.
+template <bool L2ONLY>
+__device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
                                              int nsegs, uint32_t vb, pp_super* __restrict__ table,
                                              pp_super* __restrict__ out, int final_level,
                                              const uint4* __restrict__ masks, uint32_t seg_blocks, uint32_t parity) {
@@ -231,24 +301,19 @@ __device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards
     uint32_t AW[8] = {0}, AN[8] = {0};
     // compact table: level + 1 starts at coff; the fill's children's
     // positions there are listed in slot order
-    const pp_super* tab = table + B.table + sg.coff;
     const uint32_t* htab = reinterpret_cast<const uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.coff);  // half
     const uint32_t moves = (uint32_t)(k - level);
     const uint32_t* __restrict__ rk = sg.ranks + (uint64_t)e * moves;
     auto fold = [&](uint32_t child) {
       uint32_t cW[8], cN[8];
-      if (HALF) {
-        uint32_t h[8];
-        const uint32_t* src = htab + 8 * (uint64_t)child;
-        if (L2ONLY)
-          ld256_cg(src, h);
-        else
-          ld256_nc(src, h);
-        half_unpack(h, own, cW);
-        half_unpack(h + 4, own, cN);
-      } else {
-        load_child<L2ONLY>(tab + child, cW, cN);
-      }
+      uint32_t h[8];
+      const uint32_t* src = htab + 8 * (uint64_t)child;
+      if (L2ONLY)
+        ld256_cg(src, h);
+      else
+        ld256_nc(src, h);
+      half_unpack(h, own, cW);
+      half_unpack(h + 4, own, cN);
 #pragma unroll
       for (int w = 0; w < 8; w++) AW[w] |= cW[w], AN[w] |= cN[w];
     };
@@ -287,12 +352,11 @@ __device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards
     }
   }
   if (final_level || sg.final) {
-    if (HALF) {  // the root: the wanted class, the other zero
+    // the root: the wanted class, the other zero
 #pragma unroll
-      for (int w = 0; w < 8; w++) {
-        const uint32_t K = class_bits(parity, w);
-        W[w] &= K, N[w] &= K;
-      }
+    for (int w = 0; w < 8; w++) {
+      const uint32_t K = class_bits(parity, w);
+      W[w] &= K, N[w] &= K;
     }
     store_super(out + B.out, W, N);
     return;
@@ -305,16 +369,21 @@ __device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards
   rmax(W, R);
 #pragma unroll
   for (int w = 0; w < 8; w++) P[w] |= Fo[w], R[w] |= Fo[w];
-  if (HALF) {  // on the parents' class
-    uint32_t h[8];
-    half_pack(P, own ^ 1u, h);
-    half_pack(R, own ^ 1u, h + 4);
-    st256(reinterpret_cast<uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.loff + e), h);
-  } else {
-    pp_super* r = table + B.table + sg.loff + e;
-    st256(r->win, P);
-    st256(r->notlose, R);
-  }
+  uint32_t h[8];  // on the parents' class
+  half_pack(P, own ^ 1u, h);
+  half_pack(R, own ^ 1u, h + 4);
+  st256(reinterpret_cast<uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.loff + e), h);
+}
+
+template <bool L2ONLY, bool HALF>
+__device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+                                             int nsegs, uint32_t vb, pp_super* __restrict__ table,
+                                             pp_super* __restrict__ out, int final_level,
+                                             const uint4* __restrict__ masks, uint32_t seg_blocks, uint32_t parity) {
+  if constexpr (HALF)
+    midgame_fill_half<L2ONLY>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks, parity);
+  else
+    midgame_fill_whole<L2ONLY>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks);
 }
 
 // Grid-wide barrier for a cooperative launch (every block resident).  The
