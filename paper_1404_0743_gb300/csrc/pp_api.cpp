@@ -353,6 +353,10 @@ void pp_shutdown(void) {
   cudaFree((void*)g_dev.standard);
   cudaFree((void*)g_dev.qlist);
   cudaFree((void*)g_dev.forms);
+  cudaFree((void*)g_dev.lsets);
+  cudaFree((void*)g_dev.lcover);
+  cudaFree((void*)g_dev.yrank);
+  cudaFree((void*)g_dev.qmoves);
   for (auto& kv : g_lists) cudaFree(kv.second->d_entries);
   g_lists.clear();
   g_ready = false;
@@ -634,8 +638,8 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
   // workspace: fill tables of all boards, then their five tables
   void* masks = (char*)d_workspace + (size_t)P->table_entries * fill_entry_bytes(P->parity);
   if (P->mode == 1) {
-    int rc = launch_small_and_masks(P, masks, d_out, s);
-    if (!rc && P->uses_barrier()) rc = (int)cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s);
+    int rc = P->uses_barrier() ? (int)cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s) : 0;
+    if (!rc) rc = launch_small_and_masks(P, masks, d_out, s);
     const bool half = P->parity >= 0;
     if (!rc && P->npacks)
       rc = launch_pack_persistent(P->d_boards, P->d_segs, P->d_pack_levels, (int)P->pack_levels.size(), P->d_levels,

@@ -9,33 +9,26 @@
 
 namespace pp {
 
-// Index of the last descriptor whose first block is <= b (uniform per block).
-template <typename T>
-__device__ __forceinline__ int find_block_owner(const T* __restrict__ d, int n, uint32_t b) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (d[mid].block0 <= b)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
-
-// Index of the last task whose first block is <= b: 32 probes at a time.
-template <typename T>
-__device__ __forceinline__ int find_block_owner_warp(const T* __restrict__ d, int n, uint32_t b) {
+// Index of the last descriptor whose first block (or first warp) is <= x, by
+// whole warps: 32 probes at a time, so that a thousand descriptors take two
+// dependent loads instead of ten.  x and the arguments are the same in every
+// lane; descriptor 0 starts at 0.
+template <typename T, typename First>
+__device__ __forceinline__ int find_owner(const T* __restrict__ d, int n, uint32_t x, First first) {
   const int lane = threadIdx.x & 31;
   int lo = 0;
   while (n > 1) {  // the owner is one of d[lo .. lo + n)
     const int step = (n + 31) / 32, at = lo + lane * step;
-    const bool below = lane * step < n && d[at].block0 <= b;
+    const bool below = lane * step < n && first(d[at]) <= x;
     const int last = 31 - __clz(__ballot_sync(0xFFFFFFFFu, below));  // probe 0 always holds
     n = min(step, n - last * step);
     lo += last * step;
   }
   return lo;
+}
+template <typename T>
+__device__ __forceinline__ int find_block_owner(const T* __restrict__ d, int n, uint32_t b) {
+  return find_owner(d, n, b, [](const T& t) { return t.block0; });
 }
 
 // 256-bit accesses (sm_100 and later): one load or store instruction per 32

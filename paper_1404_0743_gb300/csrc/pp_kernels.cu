@@ -1050,15 +1050,7 @@ __global__ void prepare_kernel(const pp_super* in, uint64_t n, pp_super* out) { 
 
 template <typename T>
 __device__ __forceinline__ int find_warp_owner(const T* __restrict__ d, int n, uint32_t w) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (d[mid].warp0 <= w)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
+  return find_owner(d, n, w, [](const T& t) { return t.warp0; });
 }
 
 
@@ -2062,7 +2054,7 @@ __global__ void __launch_bounds__(kTabWarps * 32, PP_TAB_MINB)
   __shared__ SecLineTask tk;
   TableSmem& sm = *reinterpret_cast<TableSmem*>(table_smem);
   if (threadIdx.x < 32) {
-    const SecLineTask* src = tasks + find_block_owner_warp(tasks, ntasks, blockIdx.x);
+    const SecLineTask* src = tasks + find_block_owner(tasks, ntasks, blockIdx.x);
     static_assert(sizeof(SecLineTask) % 4 == 0, "copied by words");
     for (int i = threadIdx.x; i < (int)(sizeof(SecLineTask) / 4); i += 32)
       reinterpret_cast<uint32_t*>(&tk)[i] = reinterpret_cast<const uint32_t*>(src)[i];

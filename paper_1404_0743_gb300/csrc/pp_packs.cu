@@ -275,7 +275,7 @@ __device__ __forceinline__ void pack_level(const MidBoard* __restrict__ boards, 
   const uint32_t per = seg_blocks & ~kSharedSegs;
   const uint32_t v1 = (uint32_t)((uint64_t)blocks * (blockIdx.x + 1) / gridDim.x);
   for (uint32_t v = (uint32_t)((uint64_t)blocks * blockIdx.x / gridDim.x); v < v1;) {
-    const uint32_t owner = per ? v / per : (uint32_t)find_block_owner_warp(segs, nsegs, v);
+    const uint32_t owner = per ? v / per : (uint32_t)find_block_owner(segs, nsegs, v);
     const uint32_t first = per ? owner * per : segs[owner].block0;
     uint32_t end = per ? first + per : owner + 1 < (uint32_t)nsegs ? segs[owner + 1].block0 : blocks;
     end = min(end, v1);
@@ -314,9 +314,21 @@ __global__ void pack_root_kernel(const MidBoard* __restrict__ boards, const MidS
   if (item < (uint32_t)npacks * 32) pack_root<HALF>(boards, segs, seg_blocks, item, table, out, parity);
 }
 
+// A level of the boards left over, the last blocks first (the packs' shares
+// of a short level fall to the first ones).  Not inlined: beside the packs'
+// code it cost the packs 7%.
+template <bool HALF>
+__device__ __noinline__ void singles_level(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+                                           const MidLevel lv, pp_super* __restrict__ table,
+                                           pp_super* __restrict__ out, int final_level,
+                                           const char* __restrict__ masks, uint32_t parity) {
+  for (uint32_t vb = gridDim.x - 1 - blockIdx.x; vb < lv.blocks; vb += gridDim.x)
+    midgame_fill<true, HALF>(boards, segs + lv.seg0, lv.nsegs, vb, table, out, final_level,
+                             reinterpret_cast<const uint4*>(masks), lv.seg_blocks, parity);
+}
+
 // All levels of a plan's packs in one cooperative launch, then the roots; the
-// boards left over one by one (singles) take their levels in the same steps
-// (an instance of its own: their code beside the packs' costs the packs 7%).
+// boards left over one by one (singles) take their levels in the same steps.
 // Children are read through L1: each is written once per launch, before the
 // grid barrier that precedes its first read, and the barrier's fence drops
 // what L1 held.
@@ -334,12 +346,8 @@ __global__ void __launch_bounds__(kPackThreads, HALF ? PP_PACK_HALF_MINB : PP_PA
       pack_level<true, HALF>(boards, segs + lv.seg0, lv.nsegs, lv.blocks, lv.seg_blocks,
                              reinterpret_cast<char*>(table), masks, parity, sg);
     }
-    if (SINGLES && L < nsingles) {
-      const MidLevel lv = singles[L];
-      for (uint32_t vb = gridDim.x - 1 - blockIdx.x; vb < lv.blocks; vb += gridDim.x)
-        midgame_fill<true, HALF>(boards, segs + lv.seg0, lv.nsegs, vb, table, out, L + 1 == nsingles,
-                                 reinterpret_cast<const uint4*>(masks), lv.seg_blocks, parity);
-    }
+    if (SINGLES && L < nsingles)
+      singles_level<HALF>(boards, segs, singles[L], table, out, L + 1 == nsingles, masks, parity);
     if (!grid_barrier(bar, status, spins)) return;
   }
   const MidLevel lv = levels[nlevels - 1];
