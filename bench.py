@@ -42,26 +42,19 @@ FILLS_PER_BOARD = 143365  # sum over m of C(12, m) C(m, ceil(m/2))
 METRIC = "boards/s (256-rotation super values)"
 # DRAM bytes (read + write) of one step of the 1024 x 12 workload, from one
 # single-pass ncu capture of the current kernels (dram__bytes_read.sum +
-# dram__bytes_write.sum): the persistent launch, and the 13 level launches of
-# the graph and per-level modes (None where a kernel has changed since)
-PERSISTENT_TRAFFIC_BYTES = 11.39e9 + 9.39e9
-LEVEL_TRAFFIC_BYTES = 10.30e9 + 9.06e9
-TRAFFIC_SOURCE = "profiles/midgame_persistent_kernel_1024x12_traffic.md"
-# what bounds the midgame kernels instead of DRAM bandwidth (ncu --set full):
-# the persistent launch on 128 boards x 12 empty cells, and one level-8
-# launch of the level kernel on 32 boards
-BINDING_LIMIT = {
-    "persistent": {"source": "profiles/midgame_persistent_kernel_128x12.md", "l1tex_throughput_pct": 71.0,
-                   "l1tex_data_pipe_pct": 70.7, "alu_pipe_pct": 49.4, "issue_active_pct": 36.2,
-                   "warps_active_pct": 49.8,
-                   "reading": "the L1 data pipe and the latency of scattered 64-byte child loads "
-                              "(long-scoreboard stalls, 12.7 per issue; grid barriers 3.1)"},
-    "level": {"source": "profiles/midgame_level_kernel_32x12.md", "l1tex_throughput_pct": 78.1,
-              "l1tex_data_pipe_pct": 70.4, "alu_pipe_pct": 53.5, "issue_active_pct": 43.0,
-              "warps_active_pct": 67.3,
-              "reading": "latency of scattered 64-byte child loads (long-scoreboard stalls, 15.7 per issue) "
-                         "and the L1 data pipe"}}
-
+# dram__bytes_write.sum), masks included: the persistent launch, and the level
+# launches of the graph and per-level modes (None where a kernel has changed
+# since)
+PERSISTENT_TRAFFIC_BYTES = 10.48e9 + 9.38e9 + 0.10e9
+LEVEL_TRAFFIC_BYTES = 10.54e9 + 8.97e9 + 0.10e9
+TRAFFIC_SOURCE = "profiles/pack_kernels_1024x12.md"
+# what bounds the pack kernels (ncu --set full, the persistent launch on 256
+# boards x 12 empty cells; the level launches run the same code)
+BINDING_LIMIT = {"source": "profiles/pack_kernels_1024x12.md", "dram_throughput_pct": 66.1,
+                 "l1tex_throughput_pct": 61.4, "alu_pipe_pct": 44.0, "issue_active_pct": 30.2,
+                 "warps_active_pct": 25.0,
+                 "reading": "latency of the children's loads at 16 warps per SM (long-scoreboard stalls, 7.3 per "
+                            "issue), DRAM at two thirds of its peak"}
 
 def peaks():
     try:
@@ -355,8 +348,8 @@ def midgame_half_run(pp, plan, ws, out, steps, warmup, stream, hbm_peak, peak_ki
         "execution": {1: "one persistent cooperative launch", 2: "one launch per level",
                       3: "CUDA graph of level launches"}[mode] + (f", {ctas} CTA/SM" if ctas else ""),
         "workspace_gb": pp.midgame_parity_workspace_bytes(BOARDS, EMPTY) / 1e9,
-        "roofline": {"bound": "hbm", "kernel": "midgame_persistent_kernel<half>" if mode == 1 else
-                     "midgame_level_kernel<half>", "achieved": alg / (ms / 1e3) / 1e9, "peak": hbm_peak,
+        "roofline": {"bound": "hbm", "kernel": "pack_persistent_kernel<half>" if mode == 1 else
+                     "pack_level_kernel<half>", "achieved": alg / (ms / 1e3) / 1e9, "peak": hbm_peak,
                      "unit": "GB/s", "frac": alg / (ms / 1e3) / 1e9 / hbm_peak, "peak_kind": peak_kind,
                      "traffic": None, "alg_bytes_per_step": alg},
     }
@@ -732,7 +725,7 @@ def d4_chain_run(pp, dev, steps, warmup, hbm_peak, peak_kind, batch_gb, host_gb)
         "ms_per_step": total_ms,
         "ms_slice36": ms[36], "ms_slice35": ms[35], "ms_slice34": ms[34],
         "value": boards / (total_ms / 1000.0), "unit": "boards/s (stored D4-reduced super values)",
-        "roofline": {"bound": "hbm", "kernel": "section_line_kernel (D4 slice 34, ready children)", "achieved": achieved,
+        "roofline": {"bound": "hbm", "kernel": "table_line_kernel (D4 slice 34, ready children)", "achieved": achieved,
                      "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "peak_kind": peak_kind,
                      "traffic": None, "alg_bytes_per_launch": bytes34},
         "slice33_stream": s33,
@@ -963,7 +956,7 @@ def run_ours(args, rank, world, local):
     gather_bytes = BOARDS * (FILLS_PER_BOARD + gathers_per_board) * 64
     launches_per_step = launches / args.steps
     achieved = alg_bytes / (ms_step / 1000.0) / 1e9
-    kernel = "midgame_persistent_kernel" if mode == 1 else "midgame_level_kernel"
+    kernel = "pack_persistent_kernel" if mode == 1 else "pack_level_kernel"
     traffic = PERSISTENT_TRAFFIC_BYTES if mode == 1 else LEVEL_TRAFFIC_BYTES
 
     # ---- end to end through the host-array entry point ------------------------
@@ -1073,7 +1066,7 @@ def run_ours(args, rank, world, local):
                      "traffic_frac": traffic / (ms_step / 1000.0) / 1e9 / hbm_peak if traffic else None,
                      "gather_bytes_per_step": gather_bytes,
                      "gather_rate_gbs": gather_bytes / (ms_step / 1000.0) / 1e9,
-                     "binding_limit": BINDING_LIMIT["persistent" if mode == 1 else "level"]},
+                     "binding_limit": BINDING_LIMIT},
         "cpu_baseline": {"value": cpu_v, "unit": "boards/s", "cores": cores, "kind": "oracle", "sample": sample},
         "e2e": {"value": e2e_value, "unit": "boards/s", "h2d_bytes_per_step": BOARDS * 8,
                 "d2h_bytes_per_step": BOARDS * 64},
