@@ -238,9 +238,11 @@ __device__ __forceinline__ void pack_root(const MidBoard* __restrict__ boards, c
   const uint32_t first = (seg_blocks & kSharedSegs) ? sg.board + pack * kPackBoards : sg.board;
   const uint32_t g1hi = row & 1, odd = row >> 1 & 1, g2hi = row >> 2;
   uint32_t w[8];
-  ld256(table + boards[first].table * kEntry + (uint64_t)sg.loff * (kEntry * kPackBoards) +
-            (HALF ? g1hi : g1hi + 2 * g2hi) * 256 + (slot + 2 * odd + 4 * group) * 32,
-        w);
+  // ordered after the last grid barrier by itself: nothing in this address
+  // was read behind the barrier, as ld256 would need
+  ld256_cg(table + boards[first].table * kEntry + (uint64_t)sg.loff * (kEntry * kPackBoards) +
+               (HALF ? g1hi : g1hi + 2 * g2hi) * 256 + (slot + 2 * odd + 4 * group) * 32,
+           w);
   if (HALF) {
 #pragma unroll
     for (int i = 0; i < 8; i++) {
