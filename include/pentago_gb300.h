@@ -315,6 +315,10 @@ void pp_server_destroy(pp_server* server);
  * section laid out as pp_slice_sections describes it); for full quadrants
  * d_child[q] is ignored.  Slice 36 takes no children (values from five in a
  * row or a tie).  d_out receives the section's dense 4-D array.
+ * Temporaries come from the device's default memory pool, in stream order, and
+ * stay in it: slice 35 the children's values a second time; below it the
+ * children's values a second time where there are at most twice as many as
+ * boards and at most 2^25 (2 GiB), without which the call is slower.
  */
 int pp_section_compute(int n, const pp_section_desc* parent, const pp_super* const d_child[4],
                        pp_super* d_out, pp_stream stream);

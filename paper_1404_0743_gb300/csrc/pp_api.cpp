@@ -1522,31 +1522,40 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
   return rc ? cuda_fail(rc, "ready children") : PP_OK;
 }
 
-// One section of slice n < 35 by lines.  Children of at most twice its boards
+// One section below slice 35 by lines.  Children of at most twice its boards
 // are first turned into ready records in a stream-ordered temporary (19 ps a
 // value), which table_line_kernel reads (27 ps a board) where the raw kernel
 // takes about 80 ps a board, and more on a small section: it has one warp for
-// 32 whole lines.
-int run_one_section(int n, SecTask tk, pp_super* out, pp_stream s) {
+// 32 whole lines.  The pool keeps what a temporary took, so its size has a
+// bound, 2 GiB (slice 36's transformed children take 3 at a step of slice
+// 35); above it children are read as they are.
+constexpr uint64_t kReadyTempValues = 1ull << 25;
+
+int run_one_section(SecTask tk, pp_super* out, pp_stream s) {
   const HostTables& t = host_tables();
-  std::vector<LineTask> kids;
+  pp_section_desc kid[4] = {};
   uint64_t total = 0, at[4] = {};
   for (int q = 0; q < 4; q++) {
     if (!(tk.movable >> q & 1)) continue;
-    pp_section_desc d{};
-    std::memcpy(d.bw, tk.bw, sizeof d.bw);
-    d.bw[q][tk.mover - 1]++;
-    for (int r = 0; r < 4; r++) d.dim[r] = (uint16_t)t.qdim[d.bw[r][0]][d.bw[r][1]];
+    std::memcpy(kid[q].bw, tk.bw, sizeof kid[q].bw);
+    kid[q].bw[q][tk.mover - 1]++;
+    for (int r = 0; r < 4; r++) kid[q].dim[r] = (uint16_t)t.qdim[kid[q].bw[r][0]][kid[q].bw[r][1]];
+    at[q] = total;
+    total += section_boards(kid[q]);
+  }
+  if (!total || total > std::min<uint64_t>(2 * tk.size, kReadyTempValues)) return run_section_lines({tk}, false, out, s);
+  std::vector<LineTask> kids;
+  for (int q = 0; q < 4; q++) {
+    if (!(tk.movable >> q & 1)) continue;
     LineTask l{};
-    if (section_boards(d) > 2 * tk.size || longest_line_task(d, &l)) return run_section_lines({tk}, false, out, s);
+    if (int rc = longest_line_task(kid[q], &l)) return rc;
     l.mover = tk.mover;  // the parents' mover
     l.child = tk.child[q];
-    l.out = at[q] = total;
-    total += section_boards(d);
+    l.out = at[q];
     kids.push_back(l);
   }
   pp_super* prep = nullptr;
-  if (!total || total > 2 * tk.size || cudaMallocAsync((void**)&prep, total * sizeof(pp_super), s) != cudaSuccess) {
+  if (cudaMallocAsync((void**)&prep, total * sizeof(pp_super), s) != cudaSuccess) {
     cudaGetLastError();  // no room for the temporary: read the children as they are
     return run_section_lines({tk}, false, out, s);
   }
@@ -1643,7 +1652,7 @@ int pp_section_compute(int n, const pp_section_desc* parent, const pp_super* con
   uint32_t blocks = 0;
   int rc = build_tasks(n, one, {0}, nullptr, d_child ? d_child : none, true, &tasks, &blocks);
   if (rc) return rc;
-  return run_one_section(n, tasks[0], d_out, s);
+  return run_one_section(tasks[0], d_out, s);
 }
 
 int pp_section_compute_desc(int n, const pp_section_desc* parent, const pp_super* const d_child[4],
