@@ -18,13 +18,18 @@
 
 // Minimum resident blocks per SM requested from the register allocator
 // (tuning knobs; 2 blocks of 256 threads cap a kernel at 128 registers, 4 at
-// 64, 6 at 40).  The midgame kernels wait on the latency of their child
-// loads: the level kernel takes as many warps as fit with few spills (6
-// blocks, 48 warps), the persistent one keeps up to four loads in flight per
-// thread at 4 (one board with 16 empty cells: 620 us; 5 blocks 624, 6 blocks
-// 633).
+// 64, 5 at 48, 6 at 40).  The midgame kernels wait on the latency of their
+// child loads.  The level kernel's lane pairs keep four loads of eight
+// registers each in flight, which 40 registers don't hold (one board with 11
+// empty cells, without allocation: 134 us at 40 registers, 119 at 48, 116 at
+// 64; fifteen with 16, graph: 6.24, 6.10 and 6.49 ms); over half tables, a
+// lane to a fill, it fits in 40.  The persistent kernel is at 4 blocks (one
+// board with 16 empty cells: 620 us; 5 blocks 624, 6 blocks 633).
 #ifndef PP_MID_MINB
-#define PP_MID_MINB 6  // midgame level kernel
+#define PP_MID_MINB 5  // midgame level kernel
+#endif
+#ifndef PP_MID_HALF_MINB
+#define PP_MID_HALF_MINB 6  // the same over half tables
 #endif
 #ifndef PP_MIDP_MINB
 #define PP_MIDP_MINB 4  // persistent midgame kernel
@@ -716,12 +721,10 @@ __global__ void __launch_bounds__(kBlock) midgame_small_kernel(const MidBoard* _
 }
 
 template <bool HALF>
-__global__ void __launch_bounds__(kBlock, PP_MID_MINB) midgame_level_kernel(const MidBoard* __restrict__ boards,
-                                                               const MidSeg* __restrict__ segs, int nsegs,
-                                                               pp_super* __restrict__ table,
-                                                               pp_super* __restrict__ out, int final_level,
-                                                               const uint4* __restrict__ masks, uint32_t seg_blocks,
-                                                               uint32_t parity) {
+__global__ void __launch_bounds__(kBlock, HALF ? PP_MID_HALF_MINB : PP_MID_MINB)
+    midgame_level_kernel(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs, int nsegs,
+                         pp_super* __restrict__ table, pp_super* __restrict__ out, int final_level,
+                         const uint4* __restrict__ masks, uint32_t seg_blocks, uint32_t parity) {
   midgame_fill<false, HALF>(boards, segs, nsegs, blockIdx.x, table, out, final_level, masks, seg_blocks, parity);
 }
 
