@@ -150,6 +150,13 @@ constexpr int kPackMinEmpty = PP_PACK_MIN_EMPTY;
 // fills in packs, 115 us against 106 all one by one; with 11, 1.6 million,
 // 160 against 169; 72 with 10, 1.1 million, the same).
 constexpr uint64_t kPackMinFills = 1250000;
+// Most fills of single boards that the persistent kernel takes by lane pairs.
+// Pairs are ahead while records come from L2 (one board with 12 empty cells 90
+// us against 112 with a lane to a fill, with 16, 10.2 million fills, 556
+// against 574; fifteen with 13 326 against 329), a lane to a fill where they
+// come from HBM (fifteen with 14, 18 million, 791 against 803; with 16, 153
+// million, 6.56 against 7.53 ms).
+constexpr uint64_t kPairFills = 12000000;
 
 std::map<std::tuple<int, int, bool>, std::unique_ptr<LevelLists>> g_lists;
 
@@ -275,6 +282,7 @@ using namespace pp;
 struct pp_midgame_plan {
   int n = 0, max_empty = 0, kmax = 0;
   uint64_t table_entries = 0;  // compact fill-table entries of all boards
+  uint64_t alone_fills = 0;    // those of the boards in `levels`
   void* d_mem = nullptr;  // one allocation holding the four arrays below
   MidBoard* d_boards = nullptr;  // the packs' boards, the ones solved one by one, the small ones
   MidSeg* d_segs = nullptr;
@@ -287,6 +295,8 @@ struct pp_midgame_plan {
   size_t small_smem = 0;
   std::vector<Level> pack_levels, levels;
   bool uses_barrier() const { return mode == 1 && (npacks || !levels.empty()); }
+  // whether the persistent kernel takes a lane pair to a fill
+  bool pairs() const { return parity < 0 && alone_fills <= kPairFills; }
   MidLevel* d_pack_levels = nullptr;
   MidLevel* d_levels = nullptr;
   uint32_t* d_sync = nullptr;  // barrier count, generation, status (persistent mode)
@@ -417,7 +427,7 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
   P->n = n;
   P->max_empty = max_empty;
   // one persistent launch (measured fastest) where the device can co-schedule it
-  P->mode = persistent_midgame_blocks(0) > 0 ? 1 : 2;
+  P->mode = persistent_midgame_blocks(0, false, false) > 0 ? 1 : 2;
   std::vector<MidBoard> boards(n);
   for (int i = 0; i < n; i++) {
     int rc = describe_board(h_boards[i], max_empty, &boards[i], i);
@@ -464,7 +474,10 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     boards[i].table = P->table_entries;  // boards' compact tables back to back
     P->table_entries += fills_total((int)boards[i].k);
     boards[i].masks = (uint64_t)i * mask_entries_per_board(max_empty);
-    if (i >= P->npacks * kPackBoards && i < nsingle) P->kmax = std::max(P->kmax, (int)boards[i].k);
+    if (i >= P->npacks * kPackBoards && i < nsingle) {
+      P->kmax = std::max(P->kmax, (int)boards[i].k);
+      P->alone_fills += fills_total((int)boards[i].k);
+    }
   }
   std::vector<MidSeg> segs;
   std::vector<SmallShape> shapes(P->nsmall ? kSmallEmpty + 1 : 0);
@@ -640,7 +653,7 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
   if (P->mode == 1) {
     int rc = P->uses_barrier() ? (int)cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s) : 0;
     if (!rc) rc = launch_small_and_masks(P, masks, d_out, s);
-    const bool half = P->parity >= 0;
+    const bool half = P->parity >= 0, pairs = P->pairs();
     if (!rc && P->npacks)
       rc = launch_pack_persistent(P->d_boards, P->d_segs, P->d_pack_levels, (int)P->pack_levels.size(), P->d_levels,
                                   (int)P->levels.size(), (pp_super*)d_workspace, d_out, P->d_sync,
@@ -648,7 +661,7 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
     else if (!rc && !P->levels.empty())
       rc = launch_midgame_persistent(P->d_boards, P->d_segs, P->d_levels, (int)P->levels.size(),
                                      (pp_super*)d_workspace, d_out, P->d_sync,
-                                     persistent_midgame_blocks(P->ctas_per_sm, half), s, masks, P->parity);
+                                     persistent_midgame_blocks(P->ctas_per_sm, half, pairs), s, masks, P->parity, pairs);
     return rc ? cuda_fail(rc, "persistent midgame launch") : PP_OK;
   }
   if (P->mode == 3) {
@@ -687,7 +700,7 @@ int pp_midgame_plan_configure(pp_midgame_plan* P, const pp_batch_opts* opts) {
   if (mode < 1 || mode > 3) return fail(PP_EINVAL, "mode %d is not 0..3", opts->persistent);
   if (opts->threads_per_block && opts->threads_per_block != kBlock)
     return fail(PP_EINVAL, "the midgame kernels run %d threads per block", kBlock);
-  if (mode == 1 && persistent_midgame_blocks(opts->ctas_per_sm, P->parity >= 0) <= 0)
+  if (mode == 1 && persistent_midgame_blocks(opts->ctas_per_sm, P->parity >= 0, P->pairs()) <= 0)
     return fail(PP_ECUDA, "persistent kernel does not fit on this device");
   P->mode = mode;
   P->ctas_per_sm = opts->ctas_per_sm;

@@ -165,6 +165,12 @@ __device__ __forceinline__ void half_unpack(const uint32_t h[4], uint32_t p, uin
   }
 }
 
+// Out of line for whole tables with a lane to a fill: beside the fold it made
+// the persistent kernel spill (one board with 16 empty cells 615 us, 584 so).
+static __device__ __noinline__ int find_segment(const MidSeg* segs, int n, uint32_t b) {
+  return find_block_owner(segs, n, b);
+}
+
 // One thread block's worth (kBlock fills) of one midgame level: block vb of
 // the level's segments (paper, "Open source and data").
 //
@@ -185,13 +191,14 @@ __device__ __forceinline__ void half_unpack(const uint32_t h[4], uint32_t p, uin
 // other way round, four loads in flight each.  A warp's load of children then
 // takes 64 bytes of each line it touches (a lane to a record took 32 at a
 // time, two L1 wavefronts a record).  Still bound by the latency and the L1
-// wavefronts of scattered records: one board with 16 empty cells 635 -> 620
-// us, 400 served queries 5.77 -> 5.49 ms.
+// wavefronts of scattered records.  Fills h0 to h1 of the block, in halves of
+// kBlock / 2.
 template <bool L2ONLY>
-__device__ __forceinline__ void midgame_fill_whole(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+__device__ __forceinline__ void midgame_fill_pairs(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
                                                   int nsegs, uint32_t vb, pp_super* __restrict__ table,
                                                   pp_super* __restrict__ out, int final_level,
-                                                  const uint4* __restrict__ masks, uint32_t seg_blocks) {
+                                                  const uint4* __restrict__ masks, uint32_t seg_blocks,
+                                                  uint32_t h0, uint32_t h1) {
   const uint32_t per = seg_blocks & ~kSharedSegs;
   const int owner = per ? (int)(vb / per) : find_block_owner(segs, nsegs, vb);
   MidSeg sg = segs[(seg_blocks & kSharedSegs) ? 0 : owner];
@@ -210,7 +217,7 @@ __device__ __forceinline__ void midgame_fill_whole(const MidBoard* __restrict__ 
       ld256_nc(kids + (uint64_t)child * sizeof(pp_super), r);
   };
 #pragma unroll 1
-  for (uint32_t half = 0; half < 2; half++) {
+  for (uint32_t half = h0; half < h1; half++) {
     const uint32_t e = (vb - sg.block0) * kBlock + half * (kBlock / 2) + (threadIdx.x >> 1);
     if (e >= sg.count) return;
     const uint64_t entry = __ldg(sg.list + e);
@@ -261,16 +268,19 @@ __device__ __forceinline__ void midgame_fill_whole(const MidBoard* __restrict__ 
   }
 }
 
-// Half tables (32-byte records): one lane to a fill.
-template <bool L2ONLY>
-__device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
+// One lane to a fill: half tables (32-byte records), and whole ones of large
+// batches in the persistent kernel (see kPairFills).
+template <bool L2ONLY, bool HALF>
+__device__ __forceinline__ void midgame_fill_lane(const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs,
                                              int nsegs, uint32_t vb, pp_super* __restrict__ table,
                                              pp_super* __restrict__ out, int final_level,
                                              const uint4* __restrict__ masks, uint32_t seg_blocks, uint32_t parity) {
   // segments of equal size (boards sharing k and mover): the owner is a division;
   // shared segments: one stored descriptor, the board follows from the owner
   const uint32_t per = seg_blocks & ~kSharedSegs;
-  const int owner = per ? (int)(vb / per) : find_block_owner(segs, nsegs, vb);
+  const int owner = per                ? (int)(vb / per)
+                    : L2ONLY && !HALF ? find_segment(segs, nsegs, vb)
+                                      : find_block_owner(segs, nsegs, vb);
   MidSeg sg = segs[(seg_blocks & kSharedSegs) ? 0 : owner];
   if (seg_blocks & kSharedSegs) sg.board += (uint32_t)owner, sg.block0 = (uint32_t)owner * per;
   const uint32_t e = (vb - sg.block0) * kBlock + threadIdx.x;
@@ -294,26 +304,33 @@ __device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ b
     uint32_t AW[8] = {0}, AN[8] = {0};
     // compact table: level + 1 starts at coff; the fill's children's
     // positions there are listed in slot order
+    const pp_super* tab = table + B.table + sg.coff;
     const uint32_t* htab = reinterpret_cast<const uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.coff);  // half
     const uint32_t moves = (uint32_t)(k - level);
     const uint32_t* __restrict__ rk = sg.ranks + (uint64_t)e * moves;
     auto fold = [&](uint32_t child) {
       uint32_t cW[8], cN[8];
-      uint32_t h[8];
-      const uint32_t* src = htab + 8 * (uint64_t)child;
-      if (L2ONLY)
-        ld256_cg(src, h);
-      else
-        ld256_nc(src, h);
-      half_unpack(h, own, cW);
-      half_unpack(h + 4, own, cN);
+      auto load = [](const void* p, uint32_t r[8]) {
+        if (L2ONLY)
+          ld256_cg(p, r);
+        else
+          ld256_nc(p, r);
+      };
+      if (HALF) {
+        uint32_t h[8];
+        load(htab + 8 * (uint64_t)child, h);
+        half_unpack(h, own, cW);
+        half_unpack(h + 4, own, cN);
+      } else {
+        load(tab[child].win, cW);
+        load(tab[child].notlose, cN);
+      }
 #pragma unroll
       for (int w = 0; w < 8; w++) AW[w] |= cW[w], AN[w] |= cN[w];
     };
     if constexpr (L2ONLY) {
-      // persistent kernel (80 registers): two moves per round, both
-      // children's loads in flight together, the next round's positions
-      // read while they are
+      // persistent kernel: two moves per round, both children's loads in
+      // flight together, the next round's positions read while they are
       uint32_t r0 = __ldg(rk), r1 = moves > 1 ? __ldg(rk + 1) : 0u;  // level < k: at least one move
       uint32_t m = 0;
       for (; m + 1 < moves; m += 2) {
@@ -325,8 +342,8 @@ __device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ b
       }
       if (m < moves) fold(r0);
     } else {
-      // level kernel (64 registers, 4 blocks per SM): one move at a time,
-      // the next move's position in flight with this child
+      // level kernel (40 registers): one move at a time, the next move's
+      // position in flight with this child
       uint32_t next = __ldg(rk);
       for (uint32_t m = 0; m < moves; m++) {
         const uint32_t child = next;
@@ -345,11 +362,12 @@ __device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ b
     }
   }
   if (final_level || sg.final) {
-    // the root: the wanted class, the other zero
+    if (HALF) {  // the root: the wanted class, the other zero
 #pragma unroll
-    for (int w = 0; w < 8; w++) {
-      const uint32_t K = class_bits(parity, w);
-      W[w] &= K, N[w] &= K;
+      for (int w = 0; w < 8; w++) {
+        const uint32_t K = class_bits(parity, w);
+        W[w] &= K, N[w] &= K;
+      }
     }
     store_super(out + B.out, W, N);
     return;
@@ -362,10 +380,16 @@ __device__ __forceinline__ void midgame_fill_half(const MidBoard* __restrict__ b
   rmax(W, R);
 #pragma unroll
   for (int w = 0; w < 8; w++) P[w] |= Fo[w], R[w] |= Fo[w];
-  uint32_t h[8];  // on the parents' class
-  half_pack(P, own ^ 1u, h);
-  half_pack(R, own ^ 1u, h + 4);
-  st256(reinterpret_cast<uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.loff + e), h);
+  if (HALF) {  // on the parents' class
+    uint32_t h[8];
+    half_pack(P, own ^ 1u, h);
+    half_pack(R, own ^ 1u, h + 4);
+    st256(reinterpret_cast<uint32_t*>(table) + 8 * ((uint64_t)B.table + sg.loff + e), h);
+  } else {
+    pp_super* r = table + B.table + sg.loff + e;
+    st256(r->win, P);
+    st256(r->notlose, R);
+  }
 }
 
 template <bool L2ONLY, bool HALF>
@@ -374,9 +398,9 @@ __device__ __forceinline__ void midgame_fill(const MidBoard* __restrict__ boards
                                              pp_super* __restrict__ out, int final_level,
                                              const uint4* __restrict__ masks, uint32_t seg_blocks, uint32_t parity) {
   if constexpr (HALF)
-    midgame_fill_half<L2ONLY>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks, parity);
+    midgame_fill_lane<L2ONLY, true>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks, parity);
   else
-    midgame_fill_whole<L2ONLY>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks);
+    midgame_fill_pairs<L2ONLY>(boards, segs, nsegs, vb, table, out, final_level, masks, seg_blocks, 0, 2);
 }
 
 // Grid-wide barrier for a cooperative launch (every block resident).  The

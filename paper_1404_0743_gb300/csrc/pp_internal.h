@@ -385,11 +385,12 @@ int launch_five_tables_packs(const MidBoard* d_boards, int npacks, int kmax, voi
 constexpr int kSlotBatch = 1024;
 int launch_five_tables_slots(const MidBoard* d_boards, const uint16_t* slots, int n, int kmax, void* d_masks,
                              pp_stream s);
-int persistent_midgame_blocks(int ctas_per_sm, bool half = false);  // co-resident blocks of the persistent kernel
+// pairs (whole tables): a lane pair to a fill, else a lane
+int persistent_midgame_blocks(int ctas_per_sm, bool half, bool pairs);  // co-resident blocks of the persistent kernel
 // d_sync: 3 words (barrier count, generation, status), zero before the launch
 int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
                               pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
-                              const void* d_masks, int parity = -1);
+                              const void* d_masks, int parity, bool pairs);
 // n boards with at most kSmallEmpty empty cells; smem: the most midgame_small_bytes of them
 int launch_midgame_small(const MidBoard* d_boards, int n, const SmallShape* d_shapes, size_t smem, pp_super* d_out,
                          int parity, pp_stream s);

@@ -24,7 +24,7 @@
 // empty cells, without allocation: 134 us at 40 registers, 119 at 48, 116 at
 // 64; fifteen with 16, graph: 6.24, 6.10 and 6.49 ms); over half tables, a
 // lane to a fill, it fits in 40.  The persistent kernel is at 4 blocks (one
-// board with 16 empty cells: 620 us; 5 blocks 624, 6 blocks 633).
+// board with 14 empty cells: 166 us; 5 blocks 185, 6 blocks 198).
 #ifndef PP_MID_MINB
 #define PP_MID_MINB 5  // midgame level kernel
 #endif
@@ -744,16 +744,26 @@ __global__ void barrier_probe_kernel(uint32_t* sync, uint32_t limit) {
 // All levels of a plan in one cooperative launch: level after level, each
 // block strides over the level's thread blocks, then the grid meets at the
 // barrier.
-template <bool HALF>
+// PAIRS (whole tables only): a lane pair to a fill, else a lane.  A lane pair's
+// block takes its kBlock fills in two halves; here each half is a visit of its
+// own, so that the blocks' fills are neighbours at any time (one board with 12
+// empty cells 111 -> 90 us, with 16 566 -> 556, fifteen with 13 336 -> 326).
+template <bool HALF, bool PAIRS>
 __global__ void __launch_bounds__(kBlock, PP_MIDP_MINB) midgame_persistent_kernel(
     const MidBoard* __restrict__ boards, const MidSeg* __restrict__ segs, const MidLevel* __restrict__ levels,
     int nlevels, pp_super* __restrict__ table, pp_super* __restrict__ out, uint32_t* bar, uint32_t* status,
     const uint4* __restrict__ masks, uint32_t parity, uint32_t spins) {
   for (int L = 0; L < nlevels; L++) {
     const MidLevel lv = levels[L];
-    for (uint32_t vb = blockIdx.x; vb < lv.blocks; vb += gridDim.x)
-      midgame_fill<true, HALF>(boards, segs + lv.seg0, lv.nsegs, vb, table, out, L + 1 == nlevels, masks,
-                               lv.seg_blocks, parity);
+    if constexpr (PAIRS) {
+      for (uint32_t v = blockIdx.x; v < 2 * lv.blocks; v += gridDim.x)  // few (kPairFills)
+        midgame_fill_pairs<true>(boards, segs + lv.seg0, lv.nsegs, v >> 1, table, out, L + 1 == nlevels, masks, lv.seg_blocks,
+                                 v & 1, (v & 1) + 1);
+    } else {
+      for (uint32_t vb = blockIdx.x; vb < lv.blocks; vb += gridDim.x)
+        midgame_fill_lane<true, HALF>(boards, segs + lv.seg0, lv.nsegs, vb, table, out, L + 1 == nlevels, masks, lv.seg_blocks,
+                                      parity);
+    }
     if (L + 1 < nlevels && !grid_barrier(bar, status, spins)) return;
   }
 }
@@ -2328,19 +2338,24 @@ int launch_five_tables_slots(const MidBoard* d_boards, const uint16_t* slots, in
   return 0;
 }
 
-int persistent_midgame_blocks(int ctas_per_sm, bool half) {
+namespace {
+const void* persistent_midgame(bool half, bool pairs) {
+  return half ? (const void*)midgame_persistent_kernel<true, false>
+              : pairs ? (const void*)midgame_persistent_kernel<false, true> : (const void*)midgame_persistent_kernel<false, false>;
+}
+}  // namespace
+
+int persistent_midgame_blocks(int ctas_per_sm, bool half, bool pairs) {
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) return 0;
-  cudaError_t e = half ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, midgame_persistent_kernel<true>, kBlock, 0)
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, midgame_persistent_kernel<false>, kBlock, 0);
-  if (e) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_midgame(half, pairs), kBlock, 0)) return 0;
   if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
   return sms * per_sm;
 }
 
 int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
                               pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
-                              const void* d_masks, int parity) {
+                              const void* d_masks, int parity, bool pairs) {
   if (grid <= 0 || nlevels <= 0 || !d_masks) return (int)cudaErrorInvalidValue;
   uint32_t* bar = d_sync;
   uint32_t* status = d_sync + 2;
@@ -2350,8 +2365,7 @@ int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, co
   void* args[] = {(void*)&d_boards, (void*)&d_segs, (void*)&d_levels, (void*)&nlevels, (void*)&d_table,
                   (void*)&d_out,    (void*)&bar,    (void*)&status,   (void*)&masks,   (void*)&p,
                   (void*)&spins};
-  const void* fn = parity >= 0 ? (const void*)midgame_persistent_kernel<true> : (const void*)midgame_persistent_kernel<false>;
-  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlock), args, 0, s);
+  cudaError_t e = cudaLaunchCooperativeKernel(persistent_midgame(parity >= 0, pairs), dim3(grid), dim3(kBlock), args, 0, s);
   count_launch();
   return (int)e;
 }
