@@ -1,0 +1,81 @@
+"""How a midgame plan arranges its boards: in packs, one by one, or both,
+beside each other or one after the other.  What was chosen is told apart by
+the launches of a run; the values are the oracle's (stored ones for 12 empty
+cells), or those of single boards a level at a time.  Bit tables, compared
+exactly."""
+import numpy as np
+import pytest
+
+from paper_1404_0743_gb300 import inputs
+from tests.gpu_helpers import midgame_oracle, ready, to_host
+from tests.test_gpu_midgame import _golden
+from tests.test_gpu_parity import class_mask
+
+pytestmark = pytest.mark.gpu
+
+
+def _stored(count):
+    """The first boards of the 1024 x 12 workload and their stored values."""
+    rows = list(_golden())[:count]
+    assert [i for i, _, _ in rows] == list(range(count))
+    return inputs.batched_midgame_boards(1024)[:count], np.array([w for _, _, w in rows], dtype=np.uint64)
+
+
+def _drawn(specs, seed):
+    return np.concatenate([inputs.midgame_boards(n, k, seed + 1000 * k) for n, k in specs])
+
+
+def _run(boards, kmax, mode, parity, launches=None):
+    import torch
+    pp = ready()
+    plan = pp.MidgamePlan(boards, kmax)
+    plan.set_parity(parity)
+    plan.configure(mode)
+    ws = torch.empty(pp.midgame_workspace_bytes(len(boards), kmax), dtype=torch.uint8, device="cuda")
+    out = torch.full((len(boards), 8), -1, dtype=torch.int64, device="cuda")
+    plan.run(ws, out)
+    before = pp.launch_count()
+    plan.run(ws, out)  # the second run finds the tables of the first
+    took = pp.launch_count() - before
+    plan.status()
+    got = to_host(out)
+    plan.close()
+    assert launches is None or took == launches
+    return got
+
+
+def _of_class(values, parity):
+    return values if parity < 0 else values & class_mask(parity)
+
+
+# launches: masks and levels of either kind (persistent: one launch of levels;
+# both kinds in one where few fills are left over), the packs' roots where a
+# level is a launch, one for the boards of at most 7 empty cells
+@pytest.fixture(scope="module")
+def shapes():
+    """Packs of two shapes, other shapes left over, boards solved in one block,
+    shuffled."""
+    twelve, values = _stored(48)
+    others = _drawn(((32, 10), (5, 9), (3, 8), (17, 6)), 0xA44A)
+    order = np.random.default_rng(9).permutation(48 + len(others))
+    return np.concatenate([twelve, others])[order], np.concatenate([values, midgame_oracle(others)])[order]
+
+
+@pytest.mark.parametrize("mode, launches", [(1, 2 + 1 + 1), (2, (1 + 13 + 1) + (1 + 10) + 1), (3, (1 + 13 + 1) + (1 + 10) + 1)])
+@pytest.mark.parametrize("parity", [-1, 0, 1])
+def test_packs_of_two_shapes_beside_single_boards(shapes, mode, launches, parity):
+    boards, want = shapes
+    assert (_run(boards, 12, mode, parity, launches) == _of_class(want, parity)).all()
+
+
+@pytest.mark.parametrize("mode, launches", [(1, 2), (2, 1 + 10 + 1), (3, 1 + 10 + 1)])
+@pytest.mark.parametrize("parity", [-1, 0, 1])
+def test_packs_of_two_shapes_alone(mode, launches, parity):
+    boards = _drawn(((16, 8), (16, 9)), 0xA44B)
+    assert (_run(boards, 9, mode, parity, launches) == _of_class(midgame_oracle(boards), parity)).all()
+
+
+@pytest.mark.parametrize("mode, launches", [(1, 2), (2, 1 + 11), (3, 1 + 11)])
+def test_single_boards_of_unequal_shapes(mode, launches):
+    boards = _drawn([(6, k) for k in (8, 9, 10)], 0xA44C)
+    assert (_run(boards, 10, mode, -1, launches) == midgame_oracle(boards)).all()
