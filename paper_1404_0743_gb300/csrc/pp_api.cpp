@@ -144,12 +144,27 @@ int describe_board(uint64_t packed, int max_empty, MidBoard* mb, int i) {
 #define PP_PACK_MIN_EMPTY 7
 #endif
 constexpr int kPackMinEmpty = PP_PACK_MIN_EMPTY;
-// Where boards are left over, a batch pays for both kinds of masks and runs
-// the single boards at the packs' occupancy, 10-20 us that fewer packed fills
-// than this don't win back (40 boards: with 10 empty cells, 0.57 million
-// fills in packs, 115 us against 106 all one by one; with 11, 1.6 million,
-// 160 against 169; 72 with 10, 1.1 million, the same).
-constexpr uint64_t kPackMinFills = 1250000;
+// Whether boards go in packs where others are left over, by the fills in packs
+// and those of the boards alone.  A batch then pays for both kinds of masks
+// and levels, which few packed fills don't win back: 40 boards with 10 empty
+// cells, 0.57 million fills in packs, take 115 us against 106 all one by one;
+// with 11, 1.6 million, 160 against 169.
+// In a persistent launch the boards left over run at the packs' occupancy
+// (whole tables), so small packs must outweigh them: 16 boards with 12 beside
+// 15 with 11 take 204 us against 208, beside 4 with 14 451 against 399, 31
+// with 12 283 against 260; from kPackAnyFills on the packs win whatever is
+// left over.  A level at a time every kind of board has its own launches: 17
+// with 12, graph, 179 us against 136, 63 with 12 356 against 370; half
+// tables 163 against 152 and 311 against 391.
+constexpr uint64_t kPackMinFills = 1250000, kPackAnyFills = 4000000;
+constexpr uint64_t kPackLevelFills = 6000000, kPackLevelHalfFills = 3000000;
+// Most fills of the boards left over that run in the packs' launch, at 16
+// warps per SM (24 for half tables) where their own kernel has 32 and its
+// grid barriers come on top: 63 boards with 12 empty cells (15 left over)
+// 403 us in one launch, 431 in two; 64 with 12 beside 4 with 14 631 against
+// 619, beside 15 with 14 1331 against 1157; 16 with 12 beside 15 with 16 9.5
+// against 7.2 ms.
+constexpr uint64_t kFusedFills = 3500000, kFusedHalfFills = 25000000;
 // Most fills of single boards that the persistent kernel takes by lane pairs.
 // Pairs are ahead while records come from L2 (one board with 12 empty cells 90
 // us against 112 with a lane to a fill, with 16, 10.2 million fills, 556
@@ -280,25 +295,43 @@ const LevelLists* level_lists(int k, int mover, std::string* err, bool grouped) 
 using namespace pp;
 
 struct pp_midgame_plan {
-  int n = 0, max_empty = 0, kmax = 0;
+  int n = 0, max_empty = 0;
   uint64_t table_entries = 0;  // compact fill-table entries of all boards
-  uint64_t alone_fills = 0;    // those of the boards in `levels`
-  void* d_mem = nullptr;  // one allocation holding the four arrays below
-  MidBoard* d_boards = nullptr;  // the packs' boards, the ones solved one by one, the small ones
-  MidSeg* d_segs = nullptr;
+  void* d_mem = nullptr;  // one allocation holding the device arrays
   using Level = MidLevel;
-  // packs of boards of one shape, and the boards left over one by one: each
-  // with its own levels, levels[j] being stones added m = kmax - j; then the
-  // boards solved in one block each
-  int npacks = 0, pack_kmax = 0, nsmall = 0;
-  const SmallShape* d_shapes = nullptr;
-  size_t small_smem = 0;
-  std::vector<Level> pack_levels, levels;
-  bool uses_barrier() const { return mode == 1 && (npacks || !levels.empty()); }
-  // whether the persistent kernel takes a lane pair to a fill
-  bool pairs() const { return parity < 0 && alone_fills <= kPairFills; }
-  MidLevel* d_pack_levels = nullptr;
-  MidLevel* d_levels = nullptr;
+  // The boards' order and levels, the device arrays in d_mem: packs of boards
+  // of one shape, and the boards left over one by one, each with its own
+  // levels, levels[j] being stones added m = kmax - j; then the boards solved
+  // in one block each.
+  struct Arrangement {
+    MidBoard* d_boards = nullptr;  // the packs' boards, the ones solved one by one, the small ones
+    MidSeg* d_segs = nullptr;
+    int npacks = 0, pack_kmax = 0, kmax = 0, nsmall = 0;
+    uint64_t alone_fills = 0;  // of the boards in `levels`
+    const SmallShape* d_shapes = nullptr;
+    size_t small_smem = 0;
+    std::vector<Level> pack_levels, levels;
+    MidLevel* d_pack_levels = nullptr;
+    MidLevel* d_levels = nullptr;
+  };
+  // every board outside packs, and in packs where whole ones can be made: both
+  // where the launch mode and the parity class decide (a one-shot plan, whose
+  // mode and class are known, holds the one it runs)
+  Arrangement arranged[2];
+  uint64_t packed_fills = 0, left_fills = 0;  // in packs where they are made, and left over
+  bool in_packs() const {
+    if (!left_fills) return true;
+    if (mode == 1)
+      return packed_fills >= kPackMinFills &&
+             (parity >= 0 || 2 * left_fills <= packed_fills || packed_fills >= kPackAnyFills);
+    return packed_fills >= (parity >= 0 ? kPackLevelHalfFills : kPackLevelFills);
+  }
+  const Arrangement& now() const { return arranged[in_packs()]; }
+  bool uses_barrier() const { return mode == 1 && (now().npacks || !now().levels.empty()); }
+  // whether the persistent kernel takes a lane pair to a fill, and whether
+  // the packs' launch takes the boards left over
+  bool pairs() const { return parity < 0 && now().alone_fills <= kPairFills; }
+  bool fused() const { return now().alone_fills <= (parity >= 0 ? kFusedHalfFills : kFusedFills); }
   uint32_t* d_sync = nullptr;  // barrier count, generation, status (persistent mode)
   int mode = 1;                // 1 persistent, 2 one launch per level, 3 graph of level launches
   int parity = -1;             // -1 every rotation; 0 / 1 only that parity class of g (half tables)
@@ -403,12 +436,12 @@ int pp_midgame_workspace_bytes(int n, int max_empty, size_t* bytes) {
 namespace pp {
 namespace {
 int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midgame_plan** plan,
-                        cudaStream_t pool_stream, bool pooled);
+                        cudaStream_t pool_stream = nullptr, bool pooled = false, int parity = -1);
 }  // namespace
 }  // namespace pp
 
 int pp_midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midgame_plan** plan) {
-  return midgame_plan_create(h_boards, n, max_empty, plan, nullptr, false);
+  return midgame_plan_create(h_boards, n, max_empty, plan);
 }
 
 }  // extern "C"
@@ -416,71 +449,72 @@ int pp_midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_mi
 namespace pp {
 namespace {
 
-int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midgame_plan** plan,
-                        cudaStream_t pool_stream, bool pooled) {
-  if (!plan) return fail(PP_EINVAL, "plan pointer is null");
-  *plan = nullptr;
-  if (!g_ready) return fail(PP_ENOTINIT, "pp_init has not run");
-  if (n < 0 || (n > 0 && !h_boards)) return fail(PP_EINVAL, "bad board array");
-  if (max_empty < 0 || max_empty > kMaxEmpty) return fail(PP_EINVAL, "max_empty %d not in 0..16", max_empty);
-  auto P = std::make_unique<pp_midgame_plan>();
-  P->n = n;
-  P->max_empty = max_empty;
-  // one persistent launch (measured fastest) where the device can co-schedule it
-  P->mode = persistent_midgame_blocks(0, false, false) > 0 ? 1 : 2;
-  std::vector<MidBoard> boards(n);
-  for (int i = 0; i < n; i++) {
-    int rc = describe_board(h_boards[i], max_empty, &boards[i], i);
-    if (rc) return rc;
-    boards[i].out = (uint64_t)i;
-  }
-  int per_k[kMaxEmpty + 1] = {};
-  for (const MidBoard& b : boards) per_k[b.k]++;
-  {
-    P->shape = "max_empty=" + std::to_string(max_empty) + " boards=";
-    for (int k = 0; k <= kMaxEmpty; k++)
-      if (per_k[k]) P->shape += std::to_string(k) + ":" + std::to_string(per_k[k]) + ",";
-  }
+// A one-shot solve runs its plan once.  A shape the autotuner has timed
+// takes the recorded mode when it is the persistent launch or the level
+// launches.  A recorded graph keeps the plan's default (one persistent
+// launch): capturing a graph for a single replay costs more than it saves,
+// and the same level launches without a graph measured slower than the
+// persistent launch (7.52 against 7.29 ms end to end for 1024 boards x 12
+// empty cells).  Untimed shapes keep the default too.
+void one_shot_mode(pp_midgame_plan* P) {
+  pp_batch_opts o;
+  if (!tune_peek(midgame_tune_key(P), &o) || o.persistent == 3) return;
+  pp_midgame_plan_configure(P, &o);  // if it fails the plan keeps its default mode
+}
+
+// Boards per number of empty cells that go in packs where packs are made.
+void pack_counts(const int per_k[kMaxEmpty + 1], int in_packs[kMaxEmpty + 1]) {
+  for (int k = 0; k <= kMaxEmpty; k++) in_packs[k] = k >= kPackMinEmpty ? per_k[k] / kPackBoards * kPackBoards : 0;
+}
+
+// Host arrays of an arrangement.
+struct ArrangedArrays {
+  std::vector<MidBoard> boards;
+  std::vector<MidSeg> segs;
+  std::vector<SmallShape> shapes;
+};
+
+// Orders the boards and lays out their levels (all but the device pointers).
+int arrange(const std::vector<MidBoard>& given, int max_empty, bool packs, pp_midgame_plan::Arrangement* A,
+            ArrangedArrays* H) {
+  const int n = (int)given.size();
+  auto& boards = H->boards;
+  auto& segs = H->segs;
+  auto& shapes = H->shapes;
   // whole packs of one shape first (the number of empty cells decides the
   // mover), then the other boards in their given order
   {
-    int taken[kMaxEmpty + 1] = {}, in_packs[kMaxEmpty + 1], first[kMaxEmpty + 1];
-    int at = 0, alone = 0;
-    uint64_t packed_fills = 0;
-    for (int k = 0; k <= kMaxEmpty; k++) {
-      in_packs[k] = k >= kPackMinEmpty ? per_k[k] / kPackBoards * kPackBoards : 0;
-      packed_fills += (uint64_t)in_packs[k] * fills_total(k);
-      if (k > kSmallEmpty) alone += per_k[k] - in_packs[k];
-    }
-    if (alone && packed_fills < kPackMinFills) std::fill(in_packs, in_packs + kMaxEmpty + 1, 0);
+    int per_k[kMaxEmpty + 1] = {}, taken[kMaxEmpty + 1] = {}, in_packs[kMaxEmpty + 1] = {}, first[kMaxEmpty + 1];
+    for (const MidBoard& b : given) per_k[b.k]++;
+    if (packs) pack_counts(per_k, in_packs);
+    int at = 0;
     for (int k = kMaxEmpty; k >= 0; k--) {
       first[k] = at;
       at += in_packs[k];
-      if (in_packs[k]) P->pack_kmax = std::max(P->pack_kmax, k);
+      if (in_packs[k]) A->pack_kmax = std::max(A->pack_kmax, k);
     }
-    P->npacks = at / kPackBoards;
-    std::vector<MidBoard> sorted(n);
+    A->npacks = at / kPackBoards;
+    boards.resize(n);
     int small = n;  // the small ones fill the end
-    for (const MidBoard& b : boards) {
+    for (const MidBoard& b : given) {
       const int k = (int)b.k;
-      sorted[taken[k] < in_packs[k] ? first[k] + taken[k] : k <= kSmallEmpty ? --small : at++] = b;
+      boards[taken[k] < in_packs[k] ? first[k] + taken[k] : k <= kSmallEmpty ? --small : at++] = b;
       taken[k]++;
     }
-    P->nsmall = n - small;
-    boards = std::move(sorted);
+    A->nsmall = n - small;
   }
-  const int nsingle = n - P->nsmall;  // where the small ones start
+  const int nsingle = n - A->nsmall;  // where the small ones start
+  uint64_t entries = 0;
   for (int i = 0; i < n; i++) {
-    boards[i].table = P->table_entries;  // boards' compact tables back to back
-    P->table_entries += fills_total((int)boards[i].k);
+    boards[i].table = entries;  // boards' compact tables back to back
+    entries += fills_total((int)boards[i].k);
     boards[i].masks = (uint64_t)i * mask_entries_per_board(max_empty);
-    if (i >= P->npacks * kPackBoards && i < nsingle) {
-      P->kmax = std::max(P->kmax, (int)boards[i].k);
-      P->alone_fills += fills_total((int)boards[i].k);
+    if (i >= A->npacks * kPackBoards && i < nsingle) {
+      A->kmax = std::max(A->kmax, (int)boards[i].k);
+      A->alone_fills += fills_total((int)boards[i].k);
     }
   }
-  std::vector<MidSeg> segs;
-  std::vector<SmallShape> shapes(P->nsmall ? kSmallEmpty + 1 : 0);
+  shapes.resize(A->nsmall ? kSmallEmpty + 1 : 0);
   {
     std::lock_guard<std::mutex> lock(g_mutex);
     for (int i = nsingle; i < n; i++) {
@@ -495,9 +529,9 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
       for (int m = 0; m <= k; m++) S.off[m] = (uint32_t)L->offset[m], S.ranks_at[m] = (uint32_t)L->ranks_at[m];
       S.off[k + 1] = (uint32_t)L->total;
       S.nranks = S.ranks_at[k];  // a full board has no moves
-      P->small_smem = std::max(P->small_smem, midgame_small_bytes(k, S.off[k + 1], S.nranks));
+      A->small_smem = std::max(A->small_smem, midgame_small_bytes(k, S.off[k + 1], S.nranks));
     }
-    if (P->small_smem > kSmallSmem) return fail(PP_ECUDA, "small boards need %zu bytes of shared memory", P->small_smem);
+    if (A->small_smem > kSmallSmem) return fail(PP_ECUDA, "small boards need %zu bytes of shared memory", A->small_smem);
     // One level's descriptors: units are packs (their first boards) or single
     // boards, `per_block` fills to a block.  When all are of one shape a
     // level has one shared descriptor, unit j being the j-th.
@@ -546,37 +580,88 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
       }
       return (int)PP_OK;
     };
-    const int packed = P->npacks * kPackBoards;
-    int rc = add_levels(0, P->npacks, kPackBoards, kPackFills, true, P->pack_kmax, &P->pack_levels);
-    if (!rc) rc = add_levels(packed, nsingle - packed, 1, kBlock, false, P->kmax, &P->levels);
+    const int packed = A->npacks * kPackBoards;
+    int rc = add_levels(0, A->npacks, kPackBoards, kPackFills, true, A->pack_kmax, &A->pack_levels);
+    if (!rc) rc = add_levels(packed, nsingle - packed, 1, kBlock, false, A->kmax, &A->levels);
     if (rc) return rc;
   }
+  return PP_OK;
+}
+
+int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midgame_plan** plan,
+                        cudaStream_t pool_stream, bool pooled, int parity) {
+  if (!plan) return fail(PP_EINVAL, "plan pointer is null");
+  *plan = nullptr;
+  if (!g_ready) return fail(PP_ENOTINIT, "pp_init has not run");
+  if (n < 0 || (n > 0 && !h_boards)) return fail(PP_EINVAL, "bad board array");
+  if (max_empty < 0 || max_empty > kMaxEmpty) return fail(PP_EINVAL, "max_empty %d not in 0..16", max_empty);
+  auto P = std::make_unique<pp_midgame_plan>();
+  P->n = n;
+  P->max_empty = max_empty;
+  P->parity = parity;
+  // one persistent launch (measured fastest) where the device can co-schedule it
+  P->mode = persistent_midgame_blocks(0, false, false) > 0 ? 1 : 2;
+  std::vector<MidBoard> boards(n);
+  int per_k[kMaxEmpty + 1] = {}, in_packs[kMaxEmpty + 1];
+  for (int i = 0; i < n; i++) {
+    int rc = describe_board(h_boards[i], max_empty, &boards[i], i);
+    if (rc) return rc;
+    boards[i].out = (uint64_t)i;
+    per_k[boards[i].k]++;
+  }
+  P->shape = "max_empty=" + std::to_string(max_empty) + " boards=";
+  pack_counts(per_k, in_packs);
+  for (int k = 0; k <= kMaxEmpty; k++) {
+    if (per_k[k]) P->shape += std::to_string(k) + ":" + std::to_string(per_k[k]) + ",";
+    P->table_entries += per_k[k] * fills_total(k);
+    P->packed_fills += in_packs[k] * fills_total(k);
+    if (k > kSmallEmpty) P->left_fills += (per_k[k] - in_packs[k]) * fills_total(k);
+  }
+  bool wanted[2] = {};
+  if (pooled) {
+    one_shot_mode(P.get());
+    wanted[P->in_packs()] = true;
+  } else {  // those of every mode and class
+    const int mode = P->mode;
+    for (P->mode = 1; P->mode <= 3; P->mode++)
+      for (P->parity = -1; P->parity <= 0; P->parity++) wanted[P->in_packs()] = true;
+    P->mode = mode;
+    P->parity = parity;
+  }
   if (n > 0) {
-    // boards, segments, levels and the barrier words (zero) packed into one
-    // allocation and one copy
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t ob = 0, os = ob + up(boards.size() * sizeof(MidBoard));
-    const size_t op = os + up(segs.size() * sizeof(MidSeg));
-    const size_t ol = op + up(P->pack_levels.size() * sizeof(MidLevel));
-    const size_t oh = ol + up(P->levels.size() * sizeof(MidLevel));
-    const size_t oy = oh + up(shapes.size() * sizeof(SmallShape)), total = oy + 4 * sizeof(uint32_t);
-    std::vector<char> pack(total, 0);
-    std::memcpy(pack.data() + ob, boards.data(), boards.size() * sizeof(MidBoard));
-    if (!segs.empty()) std::memcpy(pack.data() + os, segs.data(), segs.size() * sizeof(MidSeg));
-    if (!shapes.empty()) std::memcpy(pack.data() + oh, shapes.data(), shapes.size() * sizeof(SmallShape));
-    if (!P->pack_levels.empty())
-      std::memcpy(pack.data() + op, P->pack_levels.data(), P->pack_levels.size() * sizeof(MidLevel));
-    if (!P->levels.empty()) std::memcpy(pack.data() + ol, P->levels.data(), P->levels.size() * sizeof(MidLevel));
+    // boards, segments and levels of each arrangement and the barrier words
+    // (zero) packed into one allocation and one copy
+    std::vector<char> pack;
+    auto put = [&](const void* src, size_t bytes) {
+      const size_t at = pack.size();
+      pack.resize((at + bytes + 255) & ~(size_t)255);
+      if (bytes) std::memcpy(pack.data() + at, src, bytes);
+      return at;
+    };
+    size_t at[2][5] = {};
+    for (int p = 0; p < 2; p++) {
+      if (!wanted[p]) continue;
+      auto& A = P->arranged[p];
+      ArrangedArrays H;
+      if (int rc = arrange(boards, max_empty, p == 1, &A, &H)) return rc;
+      at[p][0] = put(H.boards.data(), H.boards.size() * sizeof(MidBoard));
+      at[p][1] = put(H.segs.data(), H.segs.size() * sizeof(MidSeg));
+      at[p][2] = put(A.pack_levels.data(), A.pack_levels.size() * sizeof(MidLevel));
+      at[p][3] = put(A.levels.data(), A.levels.size() * sizeof(MidLevel));
+      at[p][4] = put(H.shapes.data(), H.shapes.size() * sizeof(SmallShape));
+    }
+    const uint32_t zero[4] = {};
+    const size_t sync = put(zero, sizeof zero);
     cudaError_t e;
     if (pooled) {
       // stream-ordered: no device-wide synchronisation; the pageable source
       // is staged before the copy call returns
-      e = cudaMallocAsync(&P->d_mem, total, pool_stream);
-      if (!e) e = cudaMemcpyAsync(P->d_mem, pack.data(), total, cudaMemcpyHostToDevice, pool_stream);
+      e = cudaMallocAsync(&P->d_mem, pack.size(), pool_stream);
+      if (!e) e = cudaMemcpyAsync(P->d_mem, pack.data(), pack.size(), cudaMemcpyHostToDevice, pool_stream);
       if (e && P->d_mem) cudaFreeAsync(P->d_mem, pool_stream);
     } else {
-      e = cudaMalloc(&P->d_mem, total);
-      if (!e) e = cudaMemcpy(P->d_mem, pack.data(), total, cudaMemcpyHostToDevice);
+      e = cudaMalloc(&P->d_mem, pack.size());
+      if (!e) e = cudaMemcpy(P->d_mem, pack.data(), pack.size(), cudaMemcpyHostToDevice);
       if (e) cudaFree(P->d_mem);
     }
     if (e) {
@@ -586,12 +671,16 @@ int midgame_plan_create(const uint64_t* h_boards, int n, int max_empty, pp_midga
     P->pooled = pooled;
     P->pool_stream = pool_stream;
     char* base = static_cast<char*>(P->d_mem);
-    P->d_boards = reinterpret_cast<MidBoard*>(base + ob);
-    P->d_segs = reinterpret_cast<MidSeg*>(base + os);
-    P->d_pack_levels = reinterpret_cast<MidLevel*>(base + op);
-    P->d_levels = reinterpret_cast<MidLevel*>(base + ol);
-    P->d_shapes = reinterpret_cast<SmallShape*>(base + oh);
-    P->d_sync = reinterpret_cast<uint32_t*>(base + oy);
+    for (int p = 0; p < 2; p++) {
+      if (!wanted[p]) continue;
+      auto& A = P->arranged[p];
+      A.d_boards = reinterpret_cast<MidBoard*>(base + at[p][0]);
+      A.d_segs = reinterpret_cast<MidSeg*>(base + at[p][1]);
+      A.d_pack_levels = reinterpret_cast<MidLevel*>(base + at[p][2]);
+      A.d_levels = reinterpret_cast<MidLevel*>(base + at[p][3]);
+      A.d_shapes = reinterpret_cast<SmallShape*>(base + at[p][4]);
+    }
+    P->d_sync = reinterpret_cast<uint32_t*>(base + sync);
   }
   *plan = P.release();
   return PP_OK;
@@ -604,25 +693,27 @@ namespace {
 
 // The small boards, whole, and the other boards' masks.
 int launch_small_and_masks(const pp_midgame_plan* P, void* masks, pp_super* d_out, pp_stream s) {
-  const int packed = P->npacks * kPackBoards, singles = P->n - P->nsmall - packed;
-  int rc = launch_midgame_small(P->d_boards + packed + singles, P->nsmall, P->d_shapes, P->small_smem, d_out,
+  const auto& A = P->now();
+  const int packed = A.npacks * kPackBoards, singles = P->n - A.nsmall - packed;
+  int rc = launch_midgame_small(A.d_boards + packed + singles, A.nsmall, A.d_shapes, A.small_smem, d_out,
                                 P->parity, s);
-  if (!rc) rc = launch_five_tables_packs(P->d_boards, P->npacks, P->pack_kmax, masks, s);
-  if (!rc) rc = launch_five_tables(P->d_boards + packed, singles, P->kmax, masks, s);
+  if (!rc) rc = launch_five_tables_packs(A.d_boards, A.npacks, A.pack_kmax, masks, s);
+  if (!rc) rc = launch_five_tables(A.d_boards + packed, singles, A.kmax, masks, s);
   return rc;
 }
 
 // One launch per level: the packs' levels, then the other boards'.
 int launch_levels(const pp_midgame_plan* P, void* d_workspace, void* masks, pp_super* d_out, pp_stream s) {
+  const auto& A = P->now();
   int rc = launch_small_and_masks(P, masks, d_out, s);
   for (const bool packs : {true, false}) {
-    const auto& levels = packs ? P->pack_levels : P->levels;
+    const auto& levels = packs ? A.pack_levels : A.levels;
     for (size_t j = 0; !rc && j < levels.size(); j++) {
       const auto& lv = levels[j];
       const int last = j + 1 == levels.size() ? 1 : 0;
-      rc = packs ? launch_pack_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
+      rc = packs ? launch_pack_level(A.d_boards, A.d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
                                      d_out, last, s, masks, lv.seg_blocks, P->parity)
-                 : launch_midgame_level(P->d_boards, P->d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
+                 : launch_midgame_level(A.d_boards, A.d_segs + lv.seg0, lv.nsegs, lv.blocks, (pp_super*)d_workspace,
                                         d_out, last, s, masks, lv.seg_blocks, P->parity);
     }
   }
@@ -632,8 +723,9 @@ int launch_levels(const pp_midgame_plan* P, void* d_workspace, void* masks, pp_s
 // Kernels of launch_levels: masks and levels of either kind, the packs' root
 // values, and the small boards.
 uint64_t level_launches(const pp_midgame_plan* P) {
-  return (P->npacks ? P->pack_levels.size() + 2 : 0) + (P->levels.empty() ? 0 : P->levels.size() + 1) +
-         (P->nsmall ? 1 : 0);
+  const auto& A = P->now();
+  return (A.npacks ? A.pack_levels.size() + 2 : 0) + (A.levels.empty() ? 0 : A.levels.size() + 1) +
+         (A.nsmall ? 1 : 0);
 }
 
 }  // namespace
@@ -653,15 +745,16 @@ int pp_midgame_plan_run(pp_midgame_plan* P, void* d_workspace, size_t ws_bytes, 
   if (P->mode == 1) {
     int rc = P->uses_barrier() ? (int)cudaMemsetAsync(P->d_sync, 0, 4 * sizeof(uint32_t), s) : 0;
     if (!rc) rc = launch_small_and_masks(P, masks, d_out, s);
-    const bool half = P->parity >= 0, pairs = P->pairs();
-    if (!rc && P->npacks)
-      rc = launch_pack_persistent(P->d_boards, P->d_segs, P->d_pack_levels, (int)P->pack_levels.size(), P->d_levels,
-                                  (int)P->levels.size(), (pp_super*)d_workspace, d_out, P->d_sync,
-                                  persistent_pack_blocks(P->ctas_per_sm, half, !P->levels.empty()), s, masks, P->parity);
-    else if (!rc && !P->levels.empty())
-      rc = launch_midgame_persistent(P->d_boards, P->d_segs, P->d_levels, (int)P->levels.size(),
-                                     (pp_super*)d_workspace, d_out, P->d_sync,
-                                     persistent_midgame_blocks(P->ctas_per_sm, half, pairs), s, masks, P->parity, pairs);
+    const auto& A = P->now();
+    const bool half = P->parity >= 0, pairs = P->pairs(), fused = P->fused() && !A.levels.empty();
+    if (!rc && A.npacks)
+      rc = launch_pack_persistent(A.d_boards, A.d_segs, A.d_pack_levels, (int)A.pack_levels.size(), A.d_levels,
+                                  fused ? (int)A.levels.size() : 0, (pp_super*)d_workspace, d_out, P->d_sync,
+                                  persistent_pack_blocks(P->ctas_per_sm, half, fused), s, masks, P->parity);
+    if (!rc && !A.levels.empty() && !(A.npacks && fused))
+      rc = launch_midgame_persistent(A.d_boards, A.d_segs, A.d_levels, (int)A.levels.size(), (pp_super*)d_workspace,
+                                     d_out, P->d_sync, persistent_midgame_blocks(P->ctas_per_sm, half, pairs), s, masks,
+                                     P->parity, pairs);
     return rc ? cuda_fail(rc, "persistent midgame launch") : PP_OK;
   }
   if (P->mode == 3) {
@@ -812,19 +905,6 @@ int pp_midgame_parity_workspace_bytes(int n, int max_empty, size_t* bytes) {
 
 namespace {
 
-// A one-shot solve runs its plan once.  A shape the autotuner has timed
-// takes the recorded mode when it is the persistent launch or the level
-// launches.  A recorded graph keeps the plan's default (one persistent
-// launch): capturing a graph for a single replay costs more than it saves,
-// and the same level launches without a graph measured slower than the
-// persistent launch (7.52 against 7.29 ms end to end for 1024 boards x 12
-// empty cells).  Untimed shapes keep the default too.
-void one_shot_mode(pp_midgame_plan* P) {
-  pp_batch_opts o;
-  if (!tune_peek(midgame_tune_key(P), &o) || o.persistent == 3) return;
-  pp_midgame_plan_configure(P, &o);  // if it fails the plan keeps its default mode
-}
-
 int solve_device(const uint64_t* d_boards, int n, pp_super* d_out, int max_empty, int parity, void* d_workspace,
                  size_t ws_bytes, pp_stream s) {
   if (n < 0 || (n > 0 && (!d_boards || !aligned16(d_boards))))
@@ -836,11 +916,9 @@ int solve_device(const uint64_t* d_boards, int n, pp_super* d_out, int max_empty
     if (e) return cuda_fail(e, "reading boards");
   }
   pp_midgame_plan* P = nullptr;
-  int rc = midgame_plan_create(h.data(), n, max_empty, &P, s, true);
+  int rc = midgame_plan_create(h.data(), n, max_empty, &P, s, true, parity);
   if (rc) return rc;
-  rc = pp_midgame_plan_set_parity(P, parity);
-  if (!rc) one_shot_mode(P);
-  if (!rc) rc = pp_midgame_plan_run(P, d_workspace, ws_bytes, d_out, s);
+  rc = pp_midgame_plan_run(P, d_workspace, ws_bytes, d_out, s);
   uint32_t st = 0;
   cudaError_t e = cudaSuccess;
   if (!rc && P->uses_barrier()) e = cudaMemcpyAsync(&st, P->d_sync + 2, sizeof st, cudaMemcpyDeviceToHost, s);
@@ -879,7 +957,6 @@ int pp_midgame_solve_host(const uint64_t* h_boards, int n, pp_super* h_out, int 
   int rc = midgame_plan_create(h_boards, n, max_empty, &P, s, true);
   if (rc) return rc;
   pp_super* d_out = (pp_super*)((char*)d_workspace + tables);
-  one_shot_mode(P);
   rc = pp_midgame_plan_run(P, d_workspace, tables, d_out, s);
   uint32_t st = 0;
   cudaError_t e = cudaSuccess;

@@ -79,3 +79,37 @@ def test_packs_of_two_shapes_alone(mode, launches, parity):
 def test_single_boards_of_unequal_shapes(mode, launches):
     boards = _drawn([(6, k) for k in (8, 9, 10)], 0xA44C)
     assert (_run(boards, 10, mode, -1, launches) == midgame_oracle(boards)).all()
+
+
+# packed twelve-cell boards beside four with 14: 16 of them don't win their
+# second kind of levels back (whole tables), 64 do, but not with the four at
+# their occupancy
+@pytest.mark.parametrize("packed, mode, parity, launches", [
+    (16, 1, -1, 2), (16, 1, 0, 3), (16, 2, -1, 1 + 15), (16, 3, 1, 1 + 15), (64, 1, -1, 4), (64, 1, 1, 3),
+    (64, 2, -1, (1 + 13 + 1) + (1 + 15))])
+def test_choice_by_the_fills_left_over(packed, mode, parity, launches):
+    twelve, values = _stored(packed)
+    deep = _drawn(((4, 14),), 0xA44D)
+    want = np.concatenate([values, np.concatenate([_run(deep[i:i + 1], 14, 2, -1) for i in range(4)])])
+    boards = np.concatenate([deep, twelve])
+    want = np.concatenate([want[packed:], want[:packed]])
+    assert (_run(boards, 14, mode, parity, launches) == _of_class(want, parity)).all()
+
+
+def test_one_plan_through_every_mode_and_class():
+    """A plan that holds both arrangements takes each by the mode and class
+    set last."""
+    import torch
+    pp = ready()
+    twelve, values = _stored(20)  # 16 in a pack, 4 left over
+    plan = pp.MidgamePlan(twelve, 12)
+    ws = torch.empty(pp.midgame_workspace_bytes(20, 12), dtype=torch.uint8, device="cuda")
+    out = torch.zeros((20, 8), dtype=torch.int64, device="cuda")
+    for mode, parity in ((1, -1), (3, -1), (1, 0), (3, 0), (3, 1), (2, 1), (2, -1), (1, 1), (3, -1)):
+        plan.configure(mode)
+        plan.set_parity(parity)
+        out.zero_()
+        plan.run(ws, out)
+        plan.status()
+        assert (to_host(out) == _of_class(values, parity)).all()
+    plan.close()
