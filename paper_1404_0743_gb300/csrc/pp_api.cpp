@@ -136,14 +136,13 @@ int describe_board(uint64_t packed, int max_empty, MidBoard* mb, int i) {
   return PP_OK;
 }
 
-// Fewest empty cells solved in packs: from 7 on sixteen boards of one shape
-// take no longer in a pack than one by one (16 boards with 7 empty cells: 55
-// against 57 us, with 12: 145 against 179), below it a few per cent more (16
-// with 5: 41 against 38; the launch is latency there).
-#ifndef PP_PACK_MIN_EMPTY
-#define PP_PACK_MIN_EMPTY 7
-#endif
-constexpr int kPackMinEmpty = PP_PACK_MIN_EMPTY;
+// Fewest empty cells solved in packs, sixteen boards of one shape each (16
+// boards with 12 empty cells 145 us against 179 one by one).  Boards with one
+// cell fewer take a block each in shared memory, without grid barriers (600 of
+// them 28 us against 86 in packs, 3,000 114 against 142), but in packs where
+// there are so many that the barriers no longer count (6,000 202 us against
+// 220, 100,000 2.6 ms against 3.5).
+constexpr int kPackMinEmpty = kSmallEmpty + 1, kPackSmallBoards = 5000;
 // Whether boards go in packs where others are left over, by the fills in packs
 // and those of the boards alone.  A batch then pays for both kinds of masks
 // and levels, which few packed fills don't win back: 40 boards with 10 empty
@@ -464,7 +463,10 @@ void one_shot_mode(pp_midgame_plan* P) {
 
 // Boards per number of empty cells that go in packs where packs are made.
 void pack_counts(const int per_k[kMaxEmpty + 1], int in_packs[kMaxEmpty + 1]) {
-  for (int k = 0; k <= kMaxEmpty; k++) in_packs[k] = k >= kPackMinEmpty ? per_k[k] / kPackBoards * kPackBoards : 0;
+  for (int k = 0; k <= kMaxEmpty; k++) {
+    const bool packs = k >= kPackMinEmpty || (k == kSmallEmpty && per_k[k] >= kPackSmallBoards);
+    in_packs[k] = packs ? per_k[k] / kPackBoards * kPackBoards : 0;
+  }
 }
 
 // Host arrays of an arrangement.

@@ -113,3 +113,25 @@ def test_one_plan_through_every_mode_and_class():
         plan.status()
         assert (to_host(out) == _of_class(values, parity)).all()
     plan.close()
+
+
+# boards with 7 empty cells: a block each up to 4,999, packs from 5,000 on (the
+# eight left over a block each)
+@pytest.mark.parametrize("count, launches", [(16, 1), (600, 1), (4999, 1), (5000, 2 + 1)])
+def test_boards_with_seven_empty_cells(count, launches):
+    boards = inputs.midgame_boards(40, 7, 0xA44E)
+    want = midgame_oracle(boards)
+    at = np.arange(count) % 40
+    assert (_run(boards[at], 7, 1, -1, launches) == want[at]).all()
+    assert (_run(boards[at], 7, 1, 1, launches) == _of_class(want[at], 1)).all()
+
+
+# 15 boards make no pack, 16 one, 17 one and a single board (too few fills to
+# pay for both), 48 three
+@pytest.mark.parametrize("count, launches", [(15, 2), (16, 2), (17, 2), (48, 2)])
+@pytest.mark.parametrize("mode", [1, 2])
+def test_around_the_pack_size(count, launches, mode):
+    boards = inputs.midgame_boards(count, 8, 0xA44F)
+    # the packs' roots are a launch of their own where a level is one
+    level_launches = {15: 10, 16: 11, 17: 10, 48: 11}[count]
+    assert (_run(boards, 8, mode, -1, launches if mode == 1 else level_launches) == midgame_oracle(boards)).all()
