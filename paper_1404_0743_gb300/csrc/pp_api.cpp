@@ -1620,22 +1620,30 @@ int prepare_ready(int n, bool d4, const pp_super* in, const uint64_t* in_offsets
 // takes about 80 ps a board, and more on a small section: it has one warp for
 // 32 whole lines.  The pool keeps what a temporary took, so its size has a
 // bound, 2 GiB (slice 36's transformed children take 3 at a step of slice
-// 35); above it children are read as they are.
+// 35); above it children are read as they are.  So are those of a section
+// whose lines are short and few: a walk of few states ends before the second
+// launch and its uploads are paid for (9 to 4,356 boards in lines of three
+// states 26 us against 33, up to 2,200 in lines of ten 28 against 32, while
+// 162 in lines of 18 take 40).
 constexpr uint64_t kReadyTempValues = 1ull << 25;
+constexpr uint32_t kShortWalk = 4, kFewLinesWalk = 10, kFewLines = 256;
 
 int run_one_section(SecTask tk, pp_super* out, pp_stream s) {
   const HostTables& t = host_tables();
   pp_section_desc kid[4] = {};
   uint64_t total = 0, at[4] = {};
+  uint32_t walk = 0;  // states of a line
   for (int q = 0; q < 4; q++) {
     if (!(tk.movable >> q & 1)) continue;
+    walk = std::max<uint32_t>(walk, tk.dim[q]);
     std::memcpy(kid[q].bw, tk.bw, sizeof kid[q].bw);
     kid[q].bw[q][tk.mover - 1]++;
     for (int r = 0; r < 4; r++) kid[q].dim[r] = (uint16_t)t.qdim[kid[q].bw[r][0]][kid[q].bw[r][1]];
     at[q] = total;
     total += section_boards(kid[q]);
   }
-  if (!total || total > std::min<uint64_t>(2 * tk.size, kReadyTempValues)) return run_section_lines({tk}, false, out, s);
+  const bool brief = walk <= kShortWalk || (walk <= kFewLinesWalk && tk.size <= (uint64_t)walk * kFewLines);
+  if (brief || total > std::min<uint64_t>(2 * tk.size, kReadyTempValues)) return run_section_lines({tk}, false, out, s);
   std::vector<LineTask> kids;
   for (int q = 0; q < 4; q++) {
     if (!(tk.movable >> q & 1)) continue;

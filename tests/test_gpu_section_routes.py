@@ -82,3 +82,16 @@ def test_temporary_is_bounded():
 def test_children_against_boards(n, few, launches):
     _check(n, lambda boards, values, walk, lines:
            20_000 < boards < 2_000_000 and walk >= 64 and (values <= 2 * boards) == few, launches)
+
+
+# short lines, few lines of medium length; many of them, and longer ones
+@pytest.mark.parametrize("n, holds, launches", [
+    (34, lambda boards, values, walk, lines: walk == 3 and lines == 3, RAW),
+    (34, lambda boards, values, walk, lines: walk == 3 and lines > 1000, RAW),
+    (34, lambda boards, values, walk, lines: walk == 10 and 100 < lines <= 256, RAW),
+    (34, lambda boards, values, walk, lines: walk == 10 and lines > 256, READY),
+    (34, lambda boards, values, walk, lines: walk == 18 and lines < 32, READY),
+    (33, lambda boards, values, walk, lines: walk == 10 and lines < 32, RAW),
+])
+def test_short_walks_read_the_children_as_they_are(n, holds, launches):
+    _check(n, lambda boards, values, walk, lines: values <= 2 * boards and holds(boards, values, walk, lines), launches)
