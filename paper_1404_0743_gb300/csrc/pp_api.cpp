@@ -305,7 +305,7 @@ struct pp_midgame_plan {
   struct Arrangement {
     MidBoard* d_boards = nullptr;  // the packs' boards, the ones solved one by one, the small ones
     MidSeg* d_segs = nullptr;
-    int npacks = 0, pack_kmax = 0, kmax = 0, nsmall = 0;
+    int npacks = 0, pack_kmax = 0, kmax = 0, nsmall = 0, small_kmax = 0;
     uint64_t alone_fills = 0;  // of the boards in `levels`
     const SmallShape* d_shapes = nullptr;
     size_t small_smem = 0;
@@ -521,6 +521,7 @@ int arrange(const std::vector<MidBoard>& given, int max_empty, bool packs, pp_mi
     std::lock_guard<std::mutex> lock(g_mutex);
     for (int i = nsingle; i < n; i++) {
       SmallShape& S = shapes[boards[i].k];  // its number of empty cells decides the mover
+      A->small_kmax = std::max(A->small_kmax, (int)boards[i].k);
       if (S.list) continue;
       const int k = (int)boards[i].k;
       std::string err;
@@ -697,8 +698,8 @@ namespace {
 int launch_small_and_masks(const pp_midgame_plan* P, void* masks, pp_super* d_out, pp_stream s) {
   const auto& A = P->now();
   const int packed = A.npacks * kPackBoards, singles = P->n - A.nsmall - packed;
-  int rc = launch_midgame_small(A.d_boards + packed + singles, A.nsmall, A.d_shapes, A.small_smem, d_out,
-                                P->parity, s);
+  int rc = launch_midgame_small(A.d_boards + packed + singles, A.nsmall, A.small_kmax, A.d_shapes, A.small_smem,
+                                d_out, P->parity, s);
   if (!rc) rc = launch_five_tables_packs(A.d_boards, A.npacks, A.pack_kmax, masks, s);
   if (!rc) rc = launch_five_tables(A.d_boards + packed, singles, A.kmax, masks, s);
   return rc;

@@ -391,9 +391,9 @@ int persistent_midgame_blocks(int ctas_per_sm, bool half, bool pairs);  // co-re
 int launch_midgame_persistent(const MidBoard* d_boards, const MidSeg* d_segs, const MidLevel* d_levels, int nlevels,
                               pp_super* d_table, pp_super* d_out, uint32_t* d_sync, int grid, pp_stream s,
                               const void* d_masks, int parity, bool pairs);
-// n boards with at most kSmallEmpty empty cells; smem: the most midgame_small_bytes of them
-int launch_midgame_small(const MidBoard* d_boards, int n, const SmallShape* d_shapes, size_t smem, pp_super* d_out,
-                         int parity, pp_stream s);
+// n boards with at most kmax <= kSmallEmpty empty cells; smem: the most midgame_small_bytes of them
+int launch_midgame_small(const MidBoard* d_boards, int n, int kmax, const SmallShape* d_shapes, size_t smem,
+                         pp_super* d_out, int parity, pp_stream s);
 size_t midgame_small_bytes(int k, uint32_t fills, uint32_t nranks);
 // The same for packs; the final level's launch also writes the roots' values.
 int launch_pack_level(const MidBoard* d_boards, const MidSeg* d_segs, int nsegs, uint32_t blocks, pp_super* d_table,

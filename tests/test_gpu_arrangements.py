@@ -135,3 +135,12 @@ def test_around_the_pack_size(count, launches, mode):
     # the packs' roots are a launch of their own where a level is one
     level_launches = {15: 10, 16: 11, 17: 10, 48: 11}[count]
     assert (_run(boards, 8, mode, -1, launches if mode == 1 else level_launches) == midgame_oracle(boards)).all()
+
+
+# a block each, of a warp up to 4 empty cells
+@pytest.mark.parametrize("specs", [((3, 0),), ((5, 1),), ((40, 2),), ((9, 3), (2, 1)), ((70, 4),), ((7, 4), (3, 5))])
+@pytest.mark.parametrize("parity", [-1, 0, 1])
+def test_few_empty_cells(specs, parity):
+    boards = _drawn(specs, 0xA450)
+    kmax = max(k for _, k in specs)
+    assert (_run(boards, kmax, 1, parity, 1) == _of_class(midgame_oracle(boards), parity)).all()
