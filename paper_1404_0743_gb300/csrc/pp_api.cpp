@@ -149,13 +149,15 @@ constexpr int kPackMinEmpty = kSmallEmpty + 1, kPackSmallBoards = 5000;
 // cells, 0.57 million fills in packs, take 115 us against 106 all one by one;
 // with 11, 1.6 million, 160 against 169.
 // In a persistent launch the boards left over run at the packs' occupancy
-// (whole tables), so small packs must outweigh them: 16 boards with 12 beside
-// 15 with 11 take 204 us against 208, beside 4 with 14 451 against 399, 31
-// with 12 283 against 260; from kPackAnyFills on the packs win whatever is
-// left over.  A level at a time every kind of board has its own launches: 17
+// (whole tables), or after the packs, so small packs must outweigh them: 16
+// boards with 12 empty cells beside 15 with 11 take 204 us against 208, beside
+// 4 with 14 451 against 399, 31 with 12 283 against 257, 31 with 13 592
+// against 557; from kPackAnyFills on the packs win whatever is left over (64
+// with 12 beside 4 with 14 610 us against 685, beside 4 with 16 2.19 against
+// 2.27 ms).  A level at a time every kind of board has its own launches: 17
 // with 12, graph, 179 us against 136, 63 with 12 356 against 370; half
 // tables 163 against 152 and 311 against 391.
-constexpr uint64_t kPackMinFills = 1250000, kPackAnyFills = 4000000;
+constexpr uint64_t kPackMinFills = 1250000, kPackAnyFills = 8000000;
 constexpr uint64_t kPackLevelFills = 6000000, kPackLevelHalfFills = 3000000;
 // Most fills of the boards left over that run in the packs' launch, at 16
 // warps per SM (24 for half tables) where their own kernel has 32 and its

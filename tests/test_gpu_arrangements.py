@@ -96,6 +96,14 @@ def test_choice_by_the_fills_left_over(packed, mode, parity, launches):
     assert (_run(boards, 14, mode, parity, launches) == _of_class(want, parity)).all()
 
 
+# one shape, its last 15 boards left over
+@pytest.mark.parametrize("parity, launches", [(-1, 2), (0, 3)])
+def test_one_shape_with_as_many_left_over(parity, launches):
+    boards = inputs.midgame_boards(31, 13, 0xA451)
+    want = np.concatenate([_run(boards[i:i + 8], 13, 2, parity) for i in range(0, 31, 8)])
+    assert (_run(boards, 13, 1, parity, launches) == want).all()
+
+
 def test_one_plan_through_every_mode_and_class():
     """A plan that holds both arrangements takes each by the mode and class
     set last."""
