@@ -225,7 +225,8 @@ __device__ __forceinline__ void pack_fill(const PackSeg& sg, const PackWork& wor
   }
 }
 
-// The roots' values, from the sliced records into the output.  Item (pack,
+// The roots' values, from the sliced records into the output; where the same
+// launch wrote them, `table` was read after its last barrier.  Item (pack,
 // group, slot, row): byte 8 g3 + row of that table of each of eight boards,
 // row = (g1 >> 1) + 2 g2.
 template <bool HALF>
@@ -238,11 +239,9 @@ __device__ __forceinline__ void pack_root(const MidBoard* __restrict__ boards, c
   const uint32_t first = (seg_blocks & kSharedSegs) ? sg.board + pack * kPackBoards : sg.board;
   const uint32_t g1hi = row & 1, odd = row >> 1 & 1, g2hi = row >> 2;
   uint32_t w[8];
-  // ordered after the last grid barrier by itself: nothing in this address
-  // was read behind the barrier, as ld256 would need
-  ld256_cg(table + boards[first].table * kEntry + (uint64_t)sg.loff * (kEntry * kPackBoards) +
-               (HALF ? g1hi : g1hi + 2 * g2hi) * 256 + (slot + 2 * odd + 4 * group) * 32,
-           w);
+  ld256(table + boards[first].table * kEntry + (uint64_t)sg.loff * (kEntry * kPackBoards) +
+            (HALF ? g1hi : g1hi + 2 * g2hi) * 256 + (slot + 2 * odd + 4 * group) * 32,
+        w);
   if (HALF) {
 #pragma unroll
     for (int i = 0; i < 8; i++) {
@@ -352,10 +351,14 @@ __global__ void __launch_bounds__(kPackThreads, HALF ? PP_PACK_HALF_MINB : PP_PA
       singles_level<HALF>(boards, segs, singles[L], table, out, L + 1 == nsingles, masks, parity);
     if (!grid_barrier(bar, status, spins)) return;
   }
+  // the roots' addresses, too, from a load made after the last barrier (an
+  // ordered load in pack_root instead cost packs beside single boards 5%)
+  if (threadIdx.x == 0) sg.rec = reinterpret_cast<char*>(table);
+  __syncthreads();
   const MidLevel lv = levels[nlevels - 1];
   for (uint32_t item = blockIdx.x * kPackThreads + threadIdx.x; item < (uint32_t)lv.nsegs * 32;
        item += gridDim.x * kPackThreads)
-    pack_root<HALF>(boards, segs + lv.seg0, lv.seg_blocks, item, reinterpret_cast<const char*>(table), out, parity);
+    pack_root<HALF>(boards, segs + lv.seg0, lv.seg_blocks, item, sg.rec, out, parity);
 }
 
 int launch_pack_level(const MidBoard* d_boards, const MidSeg* d_segs, int nsegs, uint32_t blocks, pp_super* d_table,
