@@ -137,14 +137,19 @@ typedef struct pp_batch_opts {
  * pp_midgame_solve_host: at most
  * n (F(max_empty) 64 + 2^max_empty 64 + 64) bytes, as
  * pp_midgame_workspace_bytes gives.  Boards that share their number of empty
- * cells (7 or more) are solved sixteen at a time, their tables interleaved
- * over the room of the sixteen; the others one by one.
+ * cells (8 or more; 7 where there are at least 5,000 of them) are solved
+ * sixteen at a time, their tables interleaved over the room of the sixteen,
+ * unless other boards are left over and too few fills go in sixteens (below
+ * 1.25 to 8 million, by the fills left over, the mode and the parity class);
+ * boards with at most 7 empty cells otherwise in one thread block each, which
+ * leaves their room unused, and all others one by one.
  */
 int pp_midgame_workspace_bytes(int n, int max_empty, size_t* bytes);
 
 /* A plan: boards validated and described on the host, descriptors uploaded
- * (one allocation per plan; boards sharing their number of empty cells and
- * mover share one descriptor per level).  Running a plan is pure device
+ * (one allocation per plan, of both orders of the boards where the mode and
+ * the parity class decide between sixteens and single boards; boards sharing
+ * their number of empty cells and mover share one descriptor per level).  Running a plan is pure device
  * work on the given stream (no host synchronisation), so a run can be
  * captured in a CUDA graph.  A plan is not safe for concurrent use from
  * several threads; distinct plans are. */

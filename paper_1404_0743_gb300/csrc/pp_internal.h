@@ -210,8 +210,9 @@ struct MidLevel {
 
 // Flag in MidLevel::seg_blocks (and the seg_blocks argument of the midgame
 // kernels): the level's segments differ only in board (segment j is board
-// segs[0].board + j) and block0, so only segs[0] is stored and the kernel
-// derives the rest from the block index.
+// segs[0].board + j, of packs the pack whose first board is segs[0].board +
+// kPackBoards j) and block0, so only segs[0] is stored and the kernel derives
+// the rest from the block index.
 constexpr uint32_t kSharedSegs = 0x80000000u;
 
 // Lists of the boards solved in one block each (midgame_small_kernel), by
@@ -378,10 +379,10 @@ int launch_midgame_level(const MidBoard* d_boards, const MidSeg* d_segs, int nse
                          pp_super* d_table, pp_super* d_out, int final_level, pp_stream s, const void* d_masks,
                          uint32_t seg_blocks, int parity = -1);
 int launch_five_tables(const MidBoard* d_boards, int n, int kmax, void* d_masks, pp_stream s);
-// the same for the n boards d_boards[slots[i]] (slots: host array, passed in
-// the launches' parameters, kSlotBatch per launch)
 // the sliced masks of npacks packs, boards d_boards[16 p .. 16 p + 16)
 int launch_five_tables_packs(const MidBoard* d_boards, int npacks, int kmax, void* d_masks, pp_stream s);
+// as launch_five_tables for the n boards d_boards[slots[i]] (slots: host
+// array, passed in the launches' parameters, kSlotBatch per launch)
 constexpr int kSlotBatch = 1024;
 int launch_five_tables_slots(const MidBoard* d_boards, const uint16_t* slots, int n, int kmax, void* d_masks,
                              pp_stream s);

@@ -13,10 +13,11 @@
 // one to a lane use one sector of each line and keep the L1 data pipe the
 // bound.
 //
-// What bounds it is the children's traffic: 18.8 GB of records for 1024 boards
-// with 12 empty cells (each written and read once) take 2.8 ms at the copy
-// rate, the whole step 3.6 ms (5.5 before), of which the masks 0.19; the
-// integer pipe is a third busy, and without rmax the step takes as long.
+// What bounds it is the latency of the children's records at 16 warps per SM:
+// 18.8 GB of records for 1024 boards with 12 empty cells (each written and read
+// once) would take 2.8 ms at the copy rate, the whole step takes 3.54 (5.5
+// before), of which the masks 0.19; DRAM is two thirds busy, the integer pipe a
+// third, and without rmax the step takes as long.
 //
 // Eight lanes take one fill: two slots, two groups of eight boards, and the
 // turns g2 even and odd.  A lane holds 32 words, g0 + 4 g1 + 16 (g2 >> 1); the
